@@ -46,6 +46,15 @@ struct clean_plan_s {
   int pipe_stages = 0;
   bool tmem_allowed = true;  // CLEAN_DEBUG_MINOR_TMEM
   bool pair_allowed = true;  // CLEAN_DEBUG_MINOR_PAIR
+  // selection minor loop (minor_select.cu): the automatic choice whenever the
+  // caller leaves the group to the library
+  bool sel_ok = false;
+  int sel_G = 1;               // CTAs per tile
+  int sel_smem = 0;
+  float2* sel_boxes = nullptr; // work area of the PSF tables
+  float2* sel_h8 = nullptr;
+  float2* sel_hb = nullptr;
+  uint32_t* sel_lobe = nullptr;
   int max_rows = 0, max_w = 0;  // largest CTA slab of the minor loop
   float* psf_own = nullptr;
   bool psf_set = false;
@@ -88,7 +97,7 @@ struct clean_plan_s {
     PlanDev d;
     MinorCfg mc;
     CUtensorMap r_map, p_map, psf_map;
-    int32_t pipe, fb_path, tma, apply;
+    int32_t pipe, fb_path, tma, apply, select, sel_G, sel_smem;
   };
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t pair[2] = {nullptr, nullptr};
@@ -244,6 +253,11 @@ int check_psf(clean_plan_s* pl, cudaStream_t s) {
                                                : CLEAN_OK;
   pl->started = false;  // a run's state refers to the old PSF
   if (pl->psf_status == CLEAN_OK && (rc = fft_prepare_psf(pl, s)) != CLEAN_OK) return rc;
+  if (pl->psf_status == CLEAN_OK && pl->sel_ok) {
+    e = select_build_psf(pl->d, pl->sel_boxes, pl->sel_h8, pl->sel_hb, pl->sel_lobe, s);
+    pl->kernel_launches += 4;
+    if (e != cudaSuccess) return cuda_fail(pl, e);
+  }
   return pl->psf_status;
 }
 
@@ -289,11 +303,20 @@ bool use_pipe(const clean_plan_s* pl) {
   return !pl->mc_pipe.resident;
 }
 
-int launch_round_minor(clean_plan_s* pl, cudaStream_t s) {
+// Selection whenever the caller left the tile groups and the minor-loop
+// variant to the library.
+bool use_select(const clean_plan_s* pl) { return pl->sel_ok && pl->minor_path == 0; }
+
+// flush: the residual must hold every component after the launch (a caller
+// may look at it before the feedback).
+int launch_round_minor(clean_plan_s* pl, cudaStream_t s, bool flush) {
   const bool pipe = use_pipe(pl);
   const int ev = timed_begin(pl, 0, s);
-  cudaError_t e = launch_minor(pl->d, pipe ? pl->mc_pipe : pl->mc, pl->parity, &pl->r_map,
-                               &pl->p_map_minor, s);
+  cudaError_t e =
+      use_select(pl) ? launch_select(pl->d, pl->sel_G, pl->sel_smem, pl->parity, flush ? 1 : 0,
+                                     (uint64_t)pl->mc.spin_limit_ns, pl->mc.force_timeout, s)
+                     : launch_minor(pl->d, pipe ? pl->mc_pipe : pl->mc, pl->parity, &pl->r_map,
+                                    &pl->p_map_minor, s);
   timed_end(pl, ev, s);
   ++pl->kernel_launches;
   if (e != cudaSuccess) return cuda_fail(pl, e);
@@ -324,13 +347,18 @@ clean_plan_s::GraphKey graph_key(const clean_plan_s* pl) {
   k.fb_path = pl->feedback_path;
   k.tma = (pl->psf_map_ok && pl->feedback_path != 1) ? 1 : 0;
   k.apply = feedback_on(pl->d) ? 1 : 0;
+  k.select = use_select(pl) ? 1 : 0;
+  k.sel_G = pl->sel_G;
+  k.sel_smem = pl->sel_smem;
   return k;
 }
 
 // One round (minor loop of parity q, then its feedback) on stream s.
 cudaError_t launch_round_pair_part(const clean_plan_s* pl, const clean_plan_s::GraphKey& k,
                                    int q, cudaStream_t s) {
-  cudaError_t e = launch_minor(k.d, k.mc, q, &k.r_map, &k.p_map, s);
+  cudaError_t e = k.select ? launch_select(k.d, k.sel_G, k.sel_smem, q, 0, (uint64_t)k.mc.spin_limit_ns,
+                                           k.mc.force_timeout, s)
+                           : launch_minor(k.d, k.mc, q, &k.r_map, &k.p_map, s);
   if (e != cudaSuccess) return e;
   return launch_feedback(k.d, k.tma ? &k.psf_map : nullptr, q, k.apply,
                          (uint64_t)pl->mc.spin_limit_ns, s);
@@ -395,6 +423,8 @@ int start_run(clean_plan_s* pl, const float* d_dirty, cudaStream_t s) {
   // grid-barrier key slots start with mark bit 63 set (see exchange_keys)
   if (e == cudaSuccess)
     e = cudaMemsetAsync(pl->d.gkeys, 0x80, sizeof(uint64_t) * 4 * (size_t)pl->d.T * pl->mc.G, s);
+  if (e == cudaSuccess && pl->sel_ok)
+    e = cudaMemsetAsync(pl->d.sel.ctl, 0, sizeof(SelCtl) * (size_t)pl->d.T, s);
   if (e == cudaSuccess) e = launch_init(pl->d, d_dirty, pl->p.niter, s);
   ++pl->kernel_launches;
   if (e == cudaSuccess && pl->d.trigger > 0.f) {
@@ -495,7 +525,7 @@ int run_rounds(clean_plan_s* pl, int32_t max_rounds, cudaStream_t s) {
         }
         if (rc != -1) return rc;
       }
-      if ((rc = launch_round_minor(pl, s)) != CLEAN_OK) return rc;
+      if ((rc = launch_round_minor(pl, s, false)) != CLEAN_OK) return rc;
       if ((rc = launch_round_feedback(pl, s)) != CLEAN_OK) return rc;
       ++i;
     }
@@ -696,7 +726,7 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
     }
   }
   if (minor_prepare(mc) != cudaSuccess || (pl->pipe_ok && minor_prepare(pl->mc_pipe) != cudaSuccess) ||
-      feedback_prepare(T) != cudaSuccess) {
+      feedback_prepare(T) != cudaSuccess || select_prepare() != cudaSuccess) {
     cudaGetLastError();
     delete pl;
     return CLEAN_ERR_CUDA;
@@ -749,6 +779,14 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
     const double fft_s = (double)pl->Ly * (pl->Lx / 2 + 1) * per_cell + kFftLaunchS;
     pl->fft = fft_s < gather_s;
   }
+  SelSizes sel_z{};
+  pl->sel_ok = p->group_ctas == 0 && p->group_sync == CLEAN_SYNC_AUTO &&
+               select_geometry(&pl->d.sel, p->ny, p->nx, p->tiles_y, p->tiles_x, &sel_z);
+  pl->sel_smem = sel_z.smem;
+  // a group's CTAs share the passes over the tile: about 1024 pixels each,
+  // as far as every CTA of the launch has an SM of its own
+  pl->sel_G = (int)std::min<int64_t>(std::max(1, sms / T),
+                                     ((int64_t)maxH * maxW + 1023) / 1024);
   const size_t spec_bytes = sizeof(float2) * (size_t)pl->Ly * (pl->Lx / 2 + 1);
   const int beam_n = (2 * kMaxBeamRadius + 1) * (2 * kMaxBeamRadius + 1);
   std::vector<Req> req = {
@@ -757,6 +795,7 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
       {(void**)&pl->d.budget, sizeof(int64_t) * (size_t)T},
       {(void**)&pl->d.peak, sizeof(uint64_t) * 2 * (size_t)T},
       {(void**)&pl->d.rcount, sizeof(int32_t) * (size_t)T},
+      {(void**)&pl->d.rapplied, sizeof(int32_t) * (size_t)T},
       {(void**)&pl->d.rcomps, sizeof(clean_component) * (size_t)(cap_round * T)},
       {(void**)&pl->d.list, sizeof(clean_component) * (size_t)list_cap},
       {(void**)&pl->d.round_off, sizeof(int64_t) * (size_t)(list_cap + 1)},
@@ -776,6 +815,15 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
     req.push_back({(void**)&pl->fft_twy, sizeof(float2) * (size_t)pl->fft_ay.tw_len});
     req.push_back({(void**)&pl->fft_twx, sizeof(float2) * (size_t)pl->fft_ax.tw_len});
     req.push_back({(void**)&pl->R0, sizeof(float) * (size_t)npix});
+  }
+  if (pl->sel_ok) {
+    req.push_back({(void**)&pl->d.sel.u, sel_z.cells});
+    req.push_back({(void**)&pl->d.sel.masks, sel_z.cells});
+    req.push_back({(void**)&pl->d.sel.ctl, sel_z.ctl});
+    req.push_back({(void**)&pl->sel_boxes, sel_z.boxes});
+    req.push_back({(void**)&pl->sel_h8, sel_z.h8});
+    req.push_back({(void**)&pl->sel_hb, sel_z.hb});
+    req.push_back({(void**)&pl->sel_lobe, sel_z.lobe});
   }
   size_t total = 0;
   for (auto& r : req) total += r.bytes;
@@ -817,6 +865,11 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
   d.K = p->feedback_interval;
   d.trigger = p->feedback_trigger;
   d.cap_round = (int32_t)cap_round;
+  d.sel.h8 = pl->sel_h8;
+  d.sel.hb = pl->sel_hb;
+  d.sel.lobe = pl->sel_lobe;
+  d.sel.inside = d.cy >= maxH - 1 && d.pny - d.cy >= maxH && d.cx >= maxW - 1 &&
+                 d.pnx - d.cx >= maxW;
 
   if (pl->fft && (fft_make_twiddles(pl->fft_twy, pl->fft_ay, s) != cudaSuccess ||
                   fft_make_twiddles(pl->fft_twx, pl->fft_ax, s) != cudaSuccess)) {
@@ -824,7 +877,9 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
     clean_destroy(pl);
     return CLEAN_ERR_CUDA;
   }
-  if (cudaMemsetAsync(d.gbar, 0, sizeof(uint32_t) * T, s) != cudaSuccess ||
+  // cells past a tile's edge (row padding, smaller tiles) stay NaN: no bound
+  if ((pl->sel_ok && cudaMemsetAsync(d.sel.u, 0xff, sel_z.cells, s) != cudaSuccess) ||
+      cudaMemsetAsync(d.gbar, 0, sizeof(uint32_t) * T, s) != cudaSuccess ||
       cudaMemsetAsync(d.st, 0, sizeof(DevState), s) != cudaSuccess) {
     cudaGetLastError();
     clean_destroy(pl);
@@ -881,7 +936,7 @@ int clean_step(clean_plan_t pl, void* stream) {
   DeviceGuard g(pl->device);
   cudaStream_t s = as_stream(stream);
   if (pl->pending && (rc = launch_round_feedback(pl, s)) != CLEAN_OK) return rc;
-  return launch_round_minor(pl, s);
+  return launch_round_minor(pl, s, true);
 }
 
 int clean_feedback(clean_plan_t pl, void* stream) {
@@ -1072,6 +1127,8 @@ int clean_resume(clean_plan_t pl, const void* h_buf, int64_t bytes, void* stream
     in += sec.second;
   }
   // the grid exchange restarts its count; its key slots start marked
+  if (e == cudaSuccess && pl->sel_ok)
+    e = cudaMemsetAsync(pl->d.sel.ctl, 0, sizeof(SelCtl) * (size_t)pl->d.T, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(pl->d.gbar, 0, sizeof(uint32_t) * pl->d.T, s);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(pl->d.gkeys, 0x80, sizeof(uint64_t) * 4 * (size_t)pl->d.T * pl->mc.G, s);

@@ -82,6 +82,35 @@ struct DevState {
   int32_t pad1;
 };
 
+// Selection minor loop (minor_select.cu): components a selection may leave
+// pending, the control words of a tile's group, and a plan's tables.
+constexpr int kSelPending = 64;
+struct SelCtl {
+  unsigned long long key[2];  // peak key of a pass, by the pass's parity
+  int64_t k;                  // the posted selection: components of the round so far
+  int32_t done;               // the round is over for the tile
+  uint32_t cmd, arrived;      // selections posted / passes finished (see minor_select.cu)
+  uint32_t phases;            // passes of the tile so far in this run
+  float near;                 // the tile's resolve margin
+};
+struct SelDev {
+  float2* u;            // [T][cell_stride] bounds of R and -R per 8 x 8 cell
+  uint2* masks;         // [T][cell_stride] the cells' pixels that are candidates
+  const float2* h8;     // PSF range over the windows a cell can meet
+  const float2* hb;     // the same for a superblock of (1 << lq)^2 cells
+  const uint32_t* lobe; // exact ranges of the 8 x 8 cells around a peak
+  SelCtl* ctl;          // [T]
+  int64_t cell_stride;  // cells of the largest tile (rows of `pitch`)
+  int32_t lq, pitch;
+  int32_t oy8, ox8, w8; // h8: entry of offset box 0, row length
+  int32_t oyb, oxb, wb; // hb likewise
+  int32_t inside;       // the PSF array holds every offset between two pixels of a tile
+};
+struct SelSizes {
+  size_t cells, boxes, h8, hb, lobe, ctl;  // bytes
+  int smem;                          // dynamic shared memory of the launch
+};
+
 // Pointers and sizes every kernel of a plan sees.
 struct PlanDev {
   float* R;                 // residual, ny x nx
@@ -97,12 +126,15 @@ struct PlanDev {
   int64_t* budget;          // [T] remaining iterations per tile
   uint64_t* peak;           // [2][T] peak key per tile, indexed by round parity
   int32_t* rcount;          // [T] components of the current round per tile
+  int32_t* rapplied;        // [T] how many of them their own tile's R has had
+                            // subtracted (the feedback subtracts the rest)
   clean_component* rcomps;  // [T][cap_round] current round's components
   clean_component* list;    // [niter] all components, list order
   int64_t* round_off;       // [niter + 1] list offset of each recorded round
   uint64_t* gkeys;          // [2][T * G] per-CTA partial keys (grid sync)
   uint32_t* gbar;           // [T] grid-barrier exchanges done per tile in this run
   DevState* st;
+  SelDev sel;               // selection minor loop (sel.u null: not in use)
 };
 
 // A batched work item: tile `tile` of image `image`.
@@ -187,6 +219,22 @@ bool make_box_tensor_map(CUtensorMap* map, const float* base, int rows, int cols
 bool encode_tensor_map_2d(CUtensorMap* map, const float* base, int rows, int cols, int box_w,
                           int box_h);
 cudaError_t minor_prepare(const MinorCfg& c);  // sets function attributes
+// ---- selection minor loop (minor_select.cu) -----------------------------------
+// Table geometry and buffer sizes for an image's tiling; false if a tile is
+// too large for the packed positions.
+bool select_geometry(SelDev* g, int ny, int nx, int ty, int tx, SelSizes* z);
+// The PSF's range tables (after every PSF change); boxes: work area.
+cudaError_t select_build_psf(const PlanDev& d, float2* boxes, float2* h8, float2* hb,
+                             uint32_t* lobe, cudaStream_t s);
+cudaError_t select_prepare();  // kernel attributes
+// One round's minor loops, G CTAs a tile (G > 1: a cooperative launch); flush:
+// leave no component pending.
+cudaError_t launch_select(const PlanDev& d, int G, int smem, int parity, int flush, uint64_t limit_ns,
+                          int force_timeout, cudaStream_t s);
+// One CTA per (image, tile) item.
+cudaError_t launch_select_batch(const PlanDev* plans, const BatchItem* items, int n_items,
+                                int direct, int smem, int round, cudaStream_t s);
+
 // G CTAs per item (G = 1: independent CTAs; G > 1: one thread-block cluster
 // per item), each reading its image's plan state from `plans` (device
 // arrays); resident: each CTA's rows fit `smem` bytes of shared memory.

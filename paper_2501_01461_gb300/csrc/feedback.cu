@@ -7,7 +7,9 @@
 // (p, f) of the round that tile s != t found, in list order (tile index, then
 // iteration), R[q] <- R[q] - f * PSF[q - p + c], one rounded multiply and
 // one rounded subtract each.  This is the convolution written out term by
-// term in a fixed order, so the result is bit-reproducible.
+// term in a fixed order, so the result is bit-reproducible.  Tile t's own
+// components that its minor loop left pending (minor_select.cu) go first, as
+// they would have in a loop that subtracts each at once.
 //
 // Each CTA owns a kRows x kCols block of one tile; every thread keeps its
 // kRowsPerWarp x kColsPerLane pixels in registers for the whole component
@@ -53,6 +55,15 @@ __device__ __forceinline__ int round_total(const PlanDev& d) {
   return n;
 }
 
+// Component g of the list tile t's pixels go through (see feedback_body).
+__device__ __forceinline__ clean_component list_component(const PlanDev& d, int t, int g, int own0,
+                                                          int n_own, const int32_t* s_pre) {
+  if (g < n_own) return d.rcomps[(int64_t)t * d.cap_round + own0 + g];
+  g -= n_own;
+  const int s = find_tile(s_pre, d.T, g);
+  return d.rcomps[(int64_t)s * d.cap_round + (g - s_pre[s])];
+}
+
 // Block (bxi, byi) of tile t; blocks_x * blocks_y blocks per tile.
 __device__ __forceinline__ void feedback_body(const PlanDev& d, int parity, int apply, int t,
                                               int bxi, int byi, int blocks_x, int blocks_y) {
@@ -70,11 +81,15 @@ __device__ __forceinline__ void feedback_body(const PlanDev& d, int parity, int 
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 
   if (live) {
-    // the other tiles' components of this round, in list order
+    // the components of this round that the tile's pixels still lack, in the
+    // order they take them: its own pending ones, then the other tiles' in
+    // list order
     const bool fb = apply && feedback_on(d);  // this image feeds back at all
     for (int s = threadIdx.x; s < d.T; s += kThreads) s_cnt[s] = (s == t || !fb) ? 0 : d.rcount[s];
     block_prefix(s_cnt, s_pre, d.T);
-    const int n_other = s_pre[d.T];
+    // the tile's own pending components come first
+    const int own0 = d.rapplied[t], n_own = d.rcount[t] - own0;
+    const int n_list = n_own + s_pre[d.T];
 
     float r[kRowsPerWarp][kColsPerLane];
     bool in[kRowsPerWarp][kColsPerLane];
@@ -90,13 +105,11 @@ __device__ __forceinline__ void feedback_body(const PlanDev& d, int parity, int 
 
     const int y_first = by0 + warp * kRowsPerWarp;
     const int x_first = bx0 + lane;
-    for (int base = 0; base < n_other; base += kChunk) {
-      const int n = min(kChunk, n_other - base);
+    for (int base = 0; base < n_list; base += kChunk) {
+      const int n = min(kChunk, n_list - base);
       __syncthreads();
       for (int jj = threadIdx.x; jj < n; jj += kThreads) {
-        const int g = base + jj;
-        const int s = find_tile(s_pre, d.T, g);
-        const clean_component cc = d.rcomps[(int64_t)s * d.cap_round + (g - s_pre[s])];
+        const clean_component cc = list_component(d, t, base + jj, own0, n_own, s_pre);
         Comp4 c4;
         c4.y = cc.y;
         c4.x = cc.x;
@@ -136,7 +149,7 @@ __device__ __forceinline__ void feedback_body(const PlanDev& d, int parity, int 
         const int y = by0 + warp * kRowsPerWarp + i;
         const int x = bx0 + lane + 32 * j;
         const int gi = y * d.nx + x;
-        if (n_other > 0) d.R[(int64_t)gi] = r[i][j];
+        if (n_list > 0) d.R[(int64_t)gi] = r[i][j];
         const float a = fabsf(r[i][j]);
         if (a > best_a || (a == best_a && gi < best_i)) {
           best_a = a;
@@ -258,7 +271,8 @@ __device__ __forceinline__ void feedback_tma_body(const PlanDev& d, const CUtens
     for (int s = threadIdx.x; s < d.T; s += kThreads)
       s_cnt[s] = (s == t || !(apply && feedback_on(d))) ? 0 : d.rcount[s];
     block_prefix(s_cnt, s_pre, d.T);  // also orders the barrier set-up
-    const int n_other = s_pre[d.T];
+    const int own0 = d.rapplied[t], n_own = d.rcount[t] - own0;  // pending: first
+    const int n_list = n_own + s_pre[d.T];
 
     float r[kRowsPerWarp][kColsPerLane];
     const int y_first = by0 + warp * kRowsPerWarp;
@@ -273,13 +287,11 @@ __device__ __forceinline__ void feedback_tma_body(const PlanDev& d, const CUtens
     }
 
     int issued = 0;  // producer: loads issued so far
-    for (int cbase = 0; cbase < n_other; cbase += kListCap) {
-      const int n = min(kListCap, n_other - cbase);
+    for (int cbase = 0; cbase < n_list; cbase += kListCap) {
+      const int n = min(kListCap, n_list - cbase);
       __syncthreads();
       for (int jj = threadIdx.x; jj < n; jj += kThreads) {
-        const int g = cbase + jj;
-        const int s = find_tile(s_pre, d.T, g);
-        const clean_component cc = d.rcomps[(int64_t)s * d.cap_round + (g - s_pre[s])];
+        const clean_component cc = list_component(d, t, cbase + jj, own0, n_own, s_pre);
         const int sy0 = by0 - cc.y + d.cy;
         const int sx0 = bx0 - cc.x + d.cx;
         Win w;
@@ -361,7 +373,7 @@ __device__ __forceinline__ void feedback_tma_body(const PlanDev& d, const CUtens
           const int y = y_first + i, x = bx0 + lane + 32 * c;
           if (y >= rc.y1 || x >= rc.x1) continue;
           const int gi = y * d.nx + x;
-          if (n_other > 0) d.R[(int64_t)gi] = r[i][c];
+          if (n_list > 0) d.R[(int64_t)gi] = r[i][c];
           const float a = fabsf(r[i][c]);
           if (a > best_a || (a == best_a && gi < best_i)) {
             best_a = a;

@@ -338,6 +338,7 @@ __device__ __forceinline__ void minor_body(const PlanDev& d, const MinorCfg& c, 
   }
   if (rank == 0 && threadIdx.x == 0) {
     d.rcount[t] = (int32_t)k;
+    d.rapplied[t] = (int32_t)k;
     d.budget[t] = budget - k;
     d.gbar[t] = seq0 + (uint32_t)k;
   }
@@ -1060,6 +1061,7 @@ __device__ __forceinline__ void minor_pipe_body(const PlanDev& d, const MinorCfg
   }
   if (rank == 0 && threadIdx.x == 0) {
     d.rcount[t] = (int32_t)k;
+    d.rapplied[t] = (int32_t)k;
     d.budget[t] = budget - k;
     d.gbar[t] = seq0 + (uint32_t)k;
   }
@@ -1600,9 +1602,11 @@ __device__ __forceinline__ void minor_pair_body(const PlanDev& d, const MinorCfg
   }
   if (q == 0 && threadIdx.x == 0) {
     d.rcount[pc0.t] = (int32_t)kx0;
+    d.rapplied[pc0.t] = (int32_t)kx0;
     d.budget[pc0.t] = budget0 - kx0;
     d.gbar[pc0.t] = seq00 + (uint32_t)kx0;
     d.rcount[pc1.t] = (int32_t)kx1;
+    d.rapplied[pc1.t] = (int32_t)kx1;
     d.budget[pc1.t] = budget1 - kx1;
     d.gbar[pc1.t] = seq01 + (uint32_t)kx1;
   }

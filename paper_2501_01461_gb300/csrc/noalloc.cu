@@ -22,18 +22,19 @@ namespace cleangb {
 namespace {
 
 // Scratch layout (bytes): control block, two peak keys, the budget, the
-// component count, the grid-barrier counter, then two parity slots of
-// per-CTA partial keys (kNoAllocMaxCtas each).
+// component count, the grid-barrier counter, the applied count, then two
+// parity slots of per-CTA partial keys (kNoAllocMaxCtas each).
 constexpr int kNoAllocMaxCtas = 1024;
 constexpr size_t kOffState = 0;
 constexpr size_t kOffPeak = 256;
 constexpr size_t kOffBudget = kOffPeak + 2 * sizeof(uint64_t);
 constexpr size_t kOffCount = kOffBudget + sizeof(int64_t);
 constexpr size_t kOffBar = kOffCount + sizeof(int32_t);
+constexpr size_t kOffApplied = kOffBar + sizeof(uint32_t);
 constexpr size_t kOffKeys = 512;
 constexpr size_t kScratchBytes = kOffKeys + 2 * kNoAllocMaxCtas * sizeof(uint64_t);  // 16.5 KiB
 static_assert(sizeof(DevState) <= kOffPeak, "control block overlaps the peak keys");
-static_assert(kOffBar + sizeof(uint32_t) <= kOffKeys, "counters overlap the key slots");
+static_assert(kOffApplied + sizeof(int32_t) <= kOffKeys, "counters overlap the key slots");
 
 // The scratch.  In host code this name is only a stand-in for the symbol,
 // never a device address: the device address comes from
@@ -115,6 +116,7 @@ extern "C" CLEAN_API int clean_hogbom_noalloc(const float* d_dirty, const float*
   d.budget = reinterpret_cast<int64_t*>(base + kOffBudget);
   d.peak = reinterpret_cast<uint64_t*>(base + kOffPeak);
   d.rcount = reinterpret_cast<int32_t*>(base + kOffCount);
+  d.rapplied = reinterpret_cast<int32_t*>(base + kOffApplied);
   d.rcomps = d_comps;  // one tile, one round: the round list is the output list
   d.list = nullptr;
   d.round_off = nullptr;
