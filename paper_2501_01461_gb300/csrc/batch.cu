@@ -2,14 +2,13 @@
 // continuous batching for serving (clean_server_*).
 //
 // Every resident image's round runs in shared launches.  The minor loops of
-// all images whose residual and PSF allow 2-D TMA boxes run in ONE
-// persistent launch (one CTA per SM working through a schedule of waves:
-// each tile of each image is a unit of G CTAs in one wave, exchanging its
-// peaks through the bounded grid exchange; largest tiles first); the other
-// images' minor loops run in launches grouped by CTAs per tile and residual
-// placement (plain loads, one CTA per small tile, a thread-block cluster per
-// large one).  Then one feedback launch covers every image's blocks (two if
-// some images need the plain-load feedback).  Each image
+// all images run by selection (minor_select.cu): one CTA per tile of each
+// image, or a thread-block cluster per tile where a round needs passes over
+// the tile between selections (no feedback interval, or one above what a
+// selection holds); one launch per kind.  Tiles too large for it run the
+// plain-load loop, one CTA per small tile and one cluster per large one.  Then
+// one feedback launch covers every image's blocks (two if some images need the
+// plain-load feedback).  Each image
 // keeps its own round phase (it may have joined later), its own budgets,
 // peaks and component list, so its results are bit for bit those of its own
 // clean_plan + clean_run.  Images that finish leave the work lists; new ones
@@ -36,40 +35,26 @@ using namespace cleangb;
 namespace {
 
 constexpr int64_t kGroupSmemMax = 200 * 1024;  // resident rows per CTA
-constexpr int kMaxUnitG = 32;                   // exchange slots per tile (a pair's 2G CTAs)
-// dynamic shared memory floor of the persistent launch: above half an SM, so
-// each SM holds one CTA (units that keep residual chunks in tensor memory
-// take all of its columns)
-constexpr int kPersistSmemMin = 116 * 1024;
 
 struct Job {
   clean_plan_t plan = nullptr;
   PlanDev dev{};
   CUtensorMap map{};
   bool tma = false;
-  // residual and PSF box maps of the batched minor-loop pipeline
-  CUtensorMap rmap{}, pmap{};
-  bool pipe = false;
-  // grid-exchange slots of the persistent minor loop: 2 sets x T tiles x
-  // kMaxUnitG CTAs, owned by the engine
-  uint64_t* bkeys = nullptr;
-  // CTAs per tile in the persistent minor loop, fixed from the run's first
-  // schedule to its end: the exchange slots of tile t are t G .. t G + G - 1,
-  // and the exchange count runs on across rounds (0: not chosen yet)
-  int unit_G = 0;
-  bool unit_pair = false;  // tile pairs (fixed with unit_G: the slots are laid out by 2G)
+  int sel_smem = 0;  // dynamic shared memory of its selection (0: the plain loop)
   bool fft = false;  // feedback by FFT convolution (the job's own launches)
   int64_t id = 0;
   int slot = 0;
   bool finished = false;
 };
 
+// One launch of a round's minor loops.
 struct Group {
   int offset = 0, count = 0;  // into the item array
-  int G = 1, resident = 0, smem = 0;
-  int pipe = 0;               // 1: TMA pipeline (cfg), 0: plain loads
-  int max_rows = 0, max_w = 0;
-  MinorCfg cfg{};
+  int G = 1, smem = 0;
+  int select = 0;             // 1: selection, 0: plain loads
+  int direct = 0;             // selection without superblocks
+  int resident = 0;           // plain loads: rows in shared memory
 };
 
 }  // namespace
@@ -87,17 +72,9 @@ struct clean_engine_s {
   int items_cap = 0;
   BatchImage* d_imgs = nullptr;         // [cap] feedback geometry (TMA images first)
   CUtensorMap* d_maps = nullptr;        // [cap]
-  CUtensorMap* d_rmaps = nullptr;       // [cap] minor-loop residual boxes
-  CUtensorMap* d_pmaps = nullptr;       // [cap] minor-loop PSF boxes
   std::vector<Group> groups;
   int n_work = 0, n_tma = 0, n_gather = 0, blocks_tma = 0, blocks_plain = 0, max_T = 1;
   std::vector<int> fft_work;            // work positions of FFT-feedback jobs
-  // persistent minor loop of the pipelined images (n_waves = 0: none)
-  BatchUnitItem* d_uitems = nullptr;
-  int uitems_cap = 0;
-  int2* d_units = nullptr;
-  int units_cap = 0;
-  int n_waves = 0, p_grid = 0, p_smem = 0;
   std::vector<int> work_jobs;           // job index of each work position
   bool dirty = true;                    // work lists need a rebuild
   int round = 0;                        // rounds launched so far (global)
@@ -134,19 +111,12 @@ void engine_free(clean_engine_s* e) {
   cudaDeviceSynchronize();
   drop_graphs(e);
   if (e->cap_stream) cudaStreamDestroy(e->cap_stream);
-  for (Job& j : e->jobs) {
-    clean_destroy(j.plan);
-    cudaFree(j.bkeys);
-  }
-  cudaFree(e->d_uitems);
-  cudaFree(e->d_units);
+  for (Job& j : e->jobs) clean_destroy(j.plan);
   cudaFree(e->d_states);
   cudaFree(e->d_plans);
   cudaFree(e->d_items);
   cudaFree(e->d_imgs);
   cudaFree(e->d_maps);
-  cudaFree(e->d_rmaps);
-  cudaFree(e->d_pmaps);
   if (e->h_states) cudaFreeHost(e->h_states);
   cudaGetLastError();
   delete e;
@@ -161,9 +131,7 @@ int engine_create(clean_engine_s** out, int cap) {
       cudaMallocHost(&e->h_states, sizeof(DevState) * cap) != cudaSuccess ||
       cudaMalloc(&e->d_plans, sizeof(PlanDev) * cap) != cudaSuccess ||
       cudaMalloc(&e->d_imgs, sizeof(BatchImage) * cap) != cudaSuccess ||
-      cudaMalloc(&e->d_maps, sizeof(CUtensorMap) * cap) != cudaSuccess ||
-      cudaMalloc(&e->d_rmaps, sizeof(CUtensorMap) * cap) != cudaSuccess ||
-      cudaMalloc(&e->d_pmaps, sizeof(CUtensorMap) * cap) != cudaSuccess) {
+      cudaMalloc(&e->d_maps, sizeof(CUtensorMap) * cap) != cudaSuccess) {
     engine_free(e);
     return CLEAN_ERR_OOM;
   }
@@ -178,18 +146,14 @@ int engine_create(clean_engine_s** out, int cap) {
 int engine_start(clean_engine_s* e, Job& j, const float* d_dirty, cudaStream_t s) {
   j.dev.round0 = e->round;
   j.finished = false;
-  j.unit_G = 0;
-  j.unit_pair = false;
   cudaError_t err = cudaMemsetAsync(j.dev.st, 0, sizeof(DevState), s);
   if (err == cudaSuccess) err = cudaMemsetAsync(j.dev.peak, 0, sizeof(uint64_t) * 2 * j.dev.T, s);
   if (err == cudaSuccess) err = launch_init(j.dev, d_dirty, plan_niter(j.plan), s);
   ++e->kernel_launches;
   if (err == cudaSuccess) err = launch_first_level(j.dev, s);
   if (err == cudaSuccess && j.fft) err = plan_fft_start(j.plan, j.dev, s);
-  // the persistent minor loop's exchange slots start marked (bit 63 set), as
-  // in a single plan's run; set-up zeroed the exchange counts
-  if (err == cudaSuccess && j.bkeys)
-    err = cudaMemsetAsync(j.bkeys, 0x80, sizeof(uint64_t) * 2 * (size_t)j.dev.T * kMaxUnitG, s);
+  if (err == cudaSuccess && j.sel_smem)
+    err = cudaMemsetAsync(j.dev.sel.ctl, 0, sizeof(SelCtl) * (size_t)j.dev.T, s);
   if (err != cudaSuccess) return eng_fail(e, CLEAN_ERR_CUDA);
   std::memset(&e->h_states[j.slot], 0, sizeof(DevState));
   e->h_states[j.slot].active = 1;  // refreshed at the next status read
@@ -213,20 +177,7 @@ int engine_register(clean_engine_s* e, const clean_params* p, const float* d_psf
   j.dev = plan_device_state(j.plan);
   j.dev.st = e->d_states + j.slot;
   j.tma = plan_psf_tensor_map(j.plan, &j.map);
-  // the minor-loop pipeline needs box maps over the residual and the PSF
-  j.pipe = p->ny >= kBatchBoxRows && p->psf_ny >= kBatchBoxRows && p->nx >= kBatchBoxW &&
-           p->psf_nx >= kBatchBoxW &&
-           make_box_tensor_map(&j.pmap, d_psf, p->psf_ny, p->psf_nx, kBatchBoxW, kBatchBoxRows) &&
-           make_box_tensor_map(&j.rmap, j.dev.R, p->ny, p->nx, kBatchBoxW, kBatchBoxRows);
-  if (j.pipe) {
-    if (cudaMalloc(&j.bkeys, sizeof(uint64_t) * 2 * (size_t)j.dev.T * kMaxUnitG) != cudaSuccess) {
-      cudaGetLastError();
-      e->free_slots.push_back(j.slot);
-      clean_destroy(j.plan);
-      return CLEAN_ERR_OOM;
-    }
-    j.dev.gkeys = j.bkeys;
-  }
+  j.sel_smem = plan_select_smem(j.plan);
   j.id = e->next_id++;
   j.finished = true;  // not running until started
   e->jobs.push_back(j);
@@ -251,28 +202,16 @@ void tile_group(int h, int w, int* G, int* resident, int* smem) {
   *smem = 0;
 }
 
-// CTAs per tile for the batched pipeline: the fewest power-of-two CTAs
-// (<= 16) whose row slabs fit in shared memory beside a ring of at least two
-// PSF boxes, and, when `fast`, at least one CTA per 8192 pixels (each
-// iteration's pass stays short, as in the single-plan choice); else 16 CTAs
-// streaming their rows.  The group's geometry is checked once the group's
-// largest slab is known.
-void pipe_tile_group(int h, int w, bool fast, int* G, int* resident, int* rows) {
-  int g0 = 1;
-  while (fast && g0 < 16 && (int64_t)g0 * 8192 < (int64_t)h * w) g0 *= 2;
-  for (int g = g0; g <= 16; g *= 2) {
-    MinorCfg c;
-    const int r = (h + g - 1) / g;
-    if (minor_pipe_batch_geometry(c, g, 1, r, w)) {
-      *G = g;
-      *resident = 1;
-      *rows = r;
-      return;
-    }
-  }
-  *G = 16;
-  *resident = 0;
-  *rows = (h + 15) / 16;
+// CTAs per tile of a selection.  With at most kSelPending iterations a round
+// the tile is scanned once and the rest is one CTA's; a round of several
+// selections passes over the tile between them, which a cluster shares (about
+// 4096 pixels a CTA; at most 8, the portable cluster size).
+int select_group(const PlanDev& d) {
+  if (d.K > 0 && d.K <= kSelPending) return 1;
+  const Rect r = tile_rect(0, d.ny, d.nx, d.ty, d.tx);
+  int G = 1;
+  while (G < 8 && (int64_t)G * 4096 < (int64_t)(r.y1 - r.y0) * (r.x1 - r.x0)) G *= 2;
+  return G;
 }
 
 // Rebuilds the device work lists from the unfinished jobs.
@@ -292,145 +231,38 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
   e->work_jobs = work;
   e->max_T = 1;
   std::vector<PlanDev> plans;
-  std::vector<CUtensorMap> maps, rmaps, pmaps;
+  std::vector<CUtensorMap> maps;
   std::vector<BatchImage> imgs;
   struct Sized {
     int64_t px;
-    int pipe, G, resident, smem, rows, w;
+    int select, direct, G, resident, smem;
     BatchItem it;
   };
   std::vector<Sized> all;
   int block0 = 0;
-  // latency or throughput: when the tiles of every resident image fit on the
-  // SMs even with one CTA per 8192 pixels, use that many (short iterations);
-  // otherwise the fewest CTAs that hold each tile (the launches run in waves
-  // anyway, and fewer, larger CTAs lose less to exchanges)
-  bool fast = true;
-  {
-    int64_t ctas = 0;
-    for (int i : work) {
-      const Job& j = e->jobs[i];
-      for (int t = 0; t < j.dev.T; ++t) {
-        const Rect r = tile_rect(t, j.dev.ny, j.dev.nx, j.dev.ty, j.dev.tx);
-        int g = 1, res = 0, rows = 0, sm = 0;
-        if (j.pipe)
-          pipe_tile_group(r.y1 - r.y0, r.x1 - r.x0, true, &g, &res, &rows);
-        else
-          tile_group(r.y1 - r.y0, r.x1 - r.x0, &g, &res, &sm);
-        ctas += g;
-      }
-    }
-    int sms = 0;
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->device);
-    fast = ctas <= sms;
-  }
-  // the pipelined images' minor loops go to the persistent launch when it can
-  // be resident
-  const int p_grid = minor_batch_persistent_grid(kPersistSmemMin);
-  std::vector<BatchUnitItem> uitems;
-  std::vector<int64_t> upx;  // pixels of each unit item's tile (scheduling order)
-  int p_smem = kPersistSmemMin;
   e->blocks_tma = e->blocks_plain = 0;
   for (int w = 0; w < (int)work.size(); ++w) {
     Job& j = e->jobs[work[w]];
-    if (p_grid > 0 && j.pipe) {
-      // one G for the whole image (its tiles share the exchange slots), the
-      // largest any of its tiles asks for, kept while the run lasts
-      if (j.unit_G == 0) {
-        // tile pairs when the tile count is even and every tile is two chunks
-        // wide: G row bands per tile, each band short enough that a CTA's
-        // full chunks of both tiles sit in tensor memory (4 chunks a tile)
-        int min_w = 1 << 30, max_h = 0, half_w = 0;
-        for (int t = 0; t < j.dev.T; ++t) {
-          const Rect r = tile_rect(t, j.dev.ny, j.dev.nx, j.dev.ty, j.dev.tx);
-          min_w = std::min(min_w, r.x1 - r.x0);
-          max_h = std::max(max_h, r.y1 - r.y0);
-          half_w = std::max(half_w, ((r.x1 - r.x0) / 2 + 127) / 128 * 128);
-        }
-        const int per_band = kBatchBoxRows * std::max(1, 4 / std::max(1, half_w / 128));
-        const int Gp = (max_h + per_band - 1) / per_band;
-        if (j.dev.T % 2 == 0 && min_w >= 2 * 128 && 2 * Gp <= kMaxUnitG) {
-          j.unit_pair = true;
-          j.unit_G = Gp;
-        } else {
-          int Gi = 1;
-          for (int t = 0; t < j.dev.T; ++t) {
-            const Rect r = tile_rect(t, j.dev.ny, j.dev.nx, j.dev.ty, j.dev.tx);
-            int g = 1, res = 0, rows = 0;
-            pipe_tile_group(r.y1 - r.y0, r.x1 - r.x0, fast, &g, &res, &rows);
-            Gi = std::max(Gi, g);
-          }
-          j.unit_G = Gi;
-        }
-      }
-      const int Gi = j.unit_G;
-      if (j.unit_pair) {
-        for (int pr = 0; pr < j.dev.T / 2; ++pr) {
-          int rows = 0, wd = 0;
-          int64_t px = 0;
-          for (int t = 2 * pr; t <= 2 * pr + 1; ++t) {
-            const Rect r = tile_rect(t, j.dev.ny, j.dev.nx, j.dev.ty, j.dev.tx);
-            rows = std::max(rows, (r.y1 - r.y0 + Gi - 1) / Gi);
-            wd = std::max(wd, r.x1 - r.x0);
-            px += (int64_t)(r.y1 - r.y0) * (r.x1 - r.x0);
-          }
-          BatchUnitItem u{};
-          if (!minor_pipe_batch_geometry(u.cfg, Gi, 0, rows, wd)) return CLEAN_ERR_UNSUPPORTED;
-          u.cfg.sync = CLEAN_SYNC_GRID;
-          u.cfg.G = Gi;
-          u.cfg.pair = 1;
-          u.kind = kUnitPair;
-          u.image = w;
-          u.tile = pr;
-          u.ranks = 2 * Gi;
-          p_smem = std::max(p_smem, u.cfg.smem);
-          uitems.push_back(u);
-          upx.push_back(px);
-        }
-      }
-      for (int t = 0; t < j.dev.T && !j.unit_pair; ++t) {
-        const Rect r = tile_rect(t, j.dev.ny, j.dev.nx, j.dev.ty, j.dev.tx);
-        const int rows = (r.y1 - r.y0 + Gi - 1) / Gi, wd = r.x1 - r.x0;
-        BatchUnitItem u{};
-        if (minor_pipe_batch_geometry(u.cfg, Gi, 1, rows, wd)) {
-          u.kind = kUnitResident;
-        } else if (minor_pipe_batch_geometry(u.cfg, Gi, 0, rows, wd)) {
-          u.kind = u.cfg.tmem ? kUnitTmem : kUnitStreamed;
-        } else {
-          return CLEAN_ERR_UNSUPPORTED;
-        }
-        u.cfg.sync = CLEAN_SYNC_GRID;
-        u.cfg.G = Gi;
-        u.image = w;
-        u.tile = t;
-        u.ranks = Gi;
-        p_smem = std::max(p_smem, u.cfg.smem);
-        uitems.push_back(u);
-        upx.push_back((int64_t)(r.y1 - r.y0) * wd);
-      }
-    }
     plans.push_back(j.dev);
     maps.push_back(j.map);
-    rmaps.push_back(j.rmap);
-    pmaps.push_back(j.pmap);
     if (j.fft)
       e->fft_work.push_back(w);
     else
       ++e->n_gather;
     if (j.tma && !j.fft) ++e->n_tma;
     e->max_T = std::max(e->max_T, j.dev.T);
-    for (int t = 0; t < j.dev.T && !(p_grid > 0 && j.pipe); ++t) {
+    const int sel_G = j.sel_smem ? select_group(j.dev) : 0;
+    for (int t = 0; t < j.dev.T; ++t) {
       const Rect r = tile_rect(t, j.dev.ny, j.dev.nx, j.dev.ty, j.dev.tx);
-      Sized z;
+      Sized z{};
       z.px = (int64_t)(r.y1 - r.y0) * (r.x1 - r.x0);
-      z.pipe = j.pipe ? 1 : 0;
-      z.w = r.x1 - r.x0;
-      if (z.pipe) {
-        pipe_tile_group(r.y1 - r.y0, z.w, fast, &z.G, &z.resident, &z.rows);
-        z.smem = 0;
+      if (j.sel_smem) {
+        z.select = 1;
+        z.direct = j.dev.sel.lq == 0 ? 1 : 0;
+        z.G = sel_G;
+        z.smem = j.sel_smem;
       } else {
-        tile_group(r.y1 - r.y0, z.w, &z.G, &z.resident, &z.smem);
-        z.rows = (r.y1 - r.y0 + z.G - 1) / z.G;
+        tile_group(r.y1 - r.y0, r.x1 - r.x0, &z.G, &z.resident, &z.smem);
       }
       z.it = BatchItem{w, t};
       all.push_back(z);
@@ -449,46 +281,35 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
     }
     imgs.push_back(im);
   }
-  // groups of equal (kernel, G, resident), biggest tiles first within each
-  std::stable_sort(all.begin(), all.end(), [](const Sized& a, const Sized& b) {
-    if (a.pipe != b.pipe) return a.pipe > b.pipe;
-    if (a.G != b.G) return a.G > b.G;
-    if (a.resident != b.resident) return a.resident < b.resident;
-    return a.px > b.px;
+  // groups of one launch each, biggest tiles first within each
+  auto kind = [](const Sized& z) {
+    return ((z.select * 2 + z.direct) * 2 + z.resident) * 32 + z.G;
+  };
+  std::stable_sort(all.begin(), all.end(), [&](const Sized& a, const Sized& b) {
+    return kind(a) != kind(b) ? kind(a) > kind(b) : a.px > b.px;
   });
   e->groups.clear();
   std::vector<BatchItem> items;
   for (size_t k = 0; k < all.size(); ++k) {
-    if (e->groups.empty() || e->groups.back().pipe != all[k].pipe ||
-        e->groups.back().G != all[k].G || e->groups.back().resident != all[k].resident) {
+    if (k == 0 || kind(all[k - 1]) != kind(all[k])) {
       Group g;
       g.offset = (int)items.size();
-      g.pipe = all[k].pipe;
+      g.select = all[k].select;
+      g.direct = all[k].direct;
       g.G = all[k].G;
       g.resident = all[k].resident;
       e->groups.push_back(g);
     }
     Group& g = e->groups.back();
     g.smem = std::max(g.smem, all[k].smem);
-    g.max_rows = std::max(g.max_rows, all[k].rows);
-    g.max_w = std::max(g.max_w, all[k].w);
     ++g.count;
     items.push_back(all[k].it);
   }
-  for (Group& g : e->groups) {
-    if (g.pipe) {
-      // every tile fits alone, so the group's largest slab fits too
-      if (!minor_pipe_batch_geometry(g.cfg, g.G, g.resident, g.max_rows, g.max_w))
-        return CLEAN_ERR_UNSUPPORTED;
-      g.smem = g.cfg.smem;
-      if (g.G > 1 && minor_pipe_batch_cluster(g.G, g.resident, g.smem) != g.G)
-        return CLEAN_ERR_UNSUPPORTED;
-    } else if (g.G > 1) {
-      // a cluster size the device cannot schedule
-      const int ok = minor_batch_cluster(g.G, g.resident, g.smem);
-      if (ok != g.G) return CLEAN_ERR_UNSUPPORTED;
-    }
-  }
+  for (const Group& g : e->groups)
+    // a cluster size the device cannot schedule
+    if (g.G > 1 && !(g.select ? select_cluster_fits(g.direct, g.G, g.smem)
+                              : minor_batch_cluster(g.G, g.resident, g.smem) == g.G))
+      return CLEAN_ERR_UNSUPPORTED;
   if ((int)items.size() > e->items_cap) {
     cudaFree(e->d_items);
     e->items_cap = std::max<int>((int)items.size(), 2 * e->items_cap);
@@ -503,60 +324,12 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
       err = cudaMemcpyAsync(e->d_maps, maps.data(), sizeof(CUtensorMap) * maps.size(),
                             cudaMemcpyHostToDevice, s);
     if (err == cudaSuccess)
-      err = cudaMemcpyAsync(e->d_rmaps, rmaps.data(), sizeof(CUtensorMap) * rmaps.size(),
-                            cudaMemcpyHostToDevice, s);
-    if (err == cudaSuccess)
-      err = cudaMemcpyAsync(e->d_pmaps, pmaps.data(), sizeof(CUtensorMap) * pmaps.size(),
-                            cudaMemcpyHostToDevice, s);
-    if (err == cudaSuccess)
       err = cudaMemcpyAsync(e->d_imgs, imgs.data(), sizeof(BatchImage) * imgs.size(),
                             cudaMemcpyHostToDevice, s);
   }
   if (err == cudaSuccess && !items.empty())
     err = cudaMemcpyAsync(e->d_items, items.data(), sizeof(BatchItem) * items.size(),
                           cudaMemcpyHostToDevice, s);
-  // the persistent schedule: items largest first, each item's G ranks into
-  // the first wave with G idle CTAs (first fit)
-  std::vector<int2> units;
-  e->n_waves = 0;
-  if (!uitems.empty()) {
-    std::vector<int> order(uitems.size());
-    for (size_t i = 0; i < order.size(); ++i) order[i] = (int)i;
-    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return upx[a] > upx[b]; });
-    std::vector<int> used;  // CTAs taken in each wave
-    for (int i : order) {
-      const int G = uitems[i].ranks;
-      size_t w = 0;
-      while (w < used.size() && used[w] + G > p_grid) ++w;
-      if (w == used.size()) {
-        used.push_back(0);
-        units.resize(units.size() + p_grid, make_int2(-1, 0));
-      }
-      for (int r = 0; r < G; ++r) units[w * p_grid + used[w] + r] = make_int2(i, r);
-      used[w] += G;
-    }
-    e->n_waves = (int)used.size();
-    if ((int)uitems.size() > e->uitems_cap) {
-      cudaFree(e->d_uitems);
-      e->uitems_cap = std::max<int>((int)uitems.size(), 2 * e->uitems_cap);
-      if (cudaMalloc(&e->d_uitems, sizeof(BatchUnitItem) * e->uitems_cap) != cudaSuccess)
-        return eng_fail(e, CLEAN_ERR_OOM);
-    }
-    if ((int)units.size() > e->units_cap) {
-      cudaFree(e->d_units);
-      e->units_cap = std::max<int>((int)units.size(), 2 * e->units_cap);
-      if (cudaMalloc(&e->d_units, sizeof(int2) * e->units_cap) != cudaSuccess)
-        return eng_fail(e, CLEAN_ERR_OOM);
-    }
-    if (err == cudaSuccess)
-      err = cudaMemcpyAsync(e->d_uitems, uitems.data(), sizeof(BatchUnitItem) * uitems.size(),
-                            cudaMemcpyHostToDevice, s);
-    if (err == cudaSuccess)
-      err = cudaMemcpyAsync(e->d_units, units.data(), sizeof(int2) * units.size(),
-                            cudaMemcpyHostToDevice, s);
-  }
-  e->p_grid = p_grid;
-  e->p_smem = p_smem;
   // the host vectors die here: make the copies complete first
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);
   if (err != cudaSuccess) return eng_fail(e, CLEAN_ERR_CUDA);
@@ -578,10 +351,9 @@ int engine_read(clean_engine_s* e, cudaStream_t s) {
     // CLEANGB_REPORT_TIMEOUT: which job, tile and exchange gave up (stderr)
     if (std::getenv("CLEANGB_REPORT_TIMEOUT"))
       std::fprintf(stderr,
-                   "cleangb: timeout in job %lld (%d x %d, %d tiles, %s G %d): tile %lld, "
-                   "iteration %lld\n",
-                   (long long)j.id, j.dev.ny, j.dev.nx, j.dev.T, j.unit_pair ? "pairs" : "units",
-                   j.unit_G, (long long)(st.timeout_where >> 32),
+                   "cleangb: timeout in job %lld (%d x %d, %d tiles): tile %lld, iteration %lld\n",
+                   (long long)j.id, j.dev.ny, j.dev.nx, j.dev.T,
+                   (long long)(st.timeout_where >> 32),
                    (long long)(st.timeout_where & 0xffffffffll));
   }
   if (timeout) return eng_fail(e, CLEAN_ERR_TIMEOUT);
@@ -608,17 +380,11 @@ int engine_mark(clean_engine_s* e) {
 // The kernels of one round (round index `round`) on stream s; *n counts them.
 cudaError_t launch_round(clean_engine_s* e, int round, cudaStream_t s, int* n) {
   cudaError_t err = cudaSuccess;
-  if (e->n_waves > 0) {
-    err = launch_minor_batch_persistent(e->d_plans, e->d_uitems, e->d_units, e->n_waves,
-                                        e->p_grid, e->p_smem, e->d_rmaps, e->d_pmaps, round, s);
-    ++*n;
-    if (err != cudaSuccess) return err;
-  }
   for (const Group& g : e->groups) {
-    err = g.pipe ? launch_minor_pipe_batch(e->d_plans, e->d_items + g.offset, g.count, g.cfg,
-                                           e->d_rmaps, e->d_pmaps, round, s)
-                 : launch_minor_batch(e->d_plans, e->d_items + g.offset, g.count, g.G,
-                                      g.resident, g.smem, round, s);
+    err = g.select ? launch_select_batch(e->d_plans, e->d_items + g.offset, g.count, g.direct, g.G,
+                                         g.smem, round, 2000000000ull, s)
+                   : launch_minor_batch(e->d_plans, e->d_items + g.offset, g.count, g.G,
+                                        g.resident, g.smem, round, s);
     ++*n;
     if (err != cudaSuccess) return err;
   }
@@ -937,7 +703,6 @@ int clean_server_remove(clean_server_t sv, int64_t job_id) {
     if (e->jobs[k].id == job_id) {
       cudaDeviceSynchronize();
       clean_destroy(e->jobs[k].plan);
-      cudaFree(e->jobs[k].bkeys);
       e->free_slots.push_back(e->jobs[k].slot);
       e->jobs.erase(e->jobs.begin() + (long)k);
       e->dirty = true;

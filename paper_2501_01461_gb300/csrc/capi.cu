@@ -305,7 +305,10 @@ bool use_pipe(const clean_plan_s* pl) {
 
 // Selection whenever the caller left the tile groups and the minor-loop
 // variant to the library.
-bool use_select(const clean_plan_s* pl) { return pl->sel_ok && pl->minor_path == 0; }
+bool use_select(const clean_plan_s* pl) {
+  return pl->sel_ok && pl->minor_path == 0 && pl->p.group_ctas == 0 &&
+         pl->p.group_sync == CLEAN_SYNC_AUTO;
+}
 
 // flush: the residual must hold every component after the launch (a caller
 // may look at it before the feedback).
@@ -549,6 +552,8 @@ bool plan_psf_tensor_map(const clean_plan_s* pl, CUtensorMap* out) {
 
 int64_t plan_niter(const clean_plan_s* pl) { return pl->p.niter; }
 
+int plan_select_smem(const clean_plan_s* pl) { return pl->sel_ok ? pl->sel_smem : 0; }
+
 bool plan_uses_fft(const clean_plan_s* pl) { return pl->fft; }
 
 cudaError_t plan_fft_start(clean_plan_s* pl, const PlanDev& d, cudaStream_t s) {
@@ -780,8 +785,7 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
     pl->fft = fft_s < gather_s;
   }
   SelSizes sel_z{};
-  pl->sel_ok = p->group_ctas == 0 && p->group_sync == CLEAN_SYNC_AUTO &&
-               select_geometry(&pl->d.sel, p->ny, p->nx, p->tiles_y, p->tiles_x, &sel_z);
+  pl->sel_ok = select_geometry(&pl->d.sel, p->ny, p->nx, p->tiles_y, p->tiles_x, &sel_z);
   pl->sel_smem = sel_z.smem;
   // a group's CTAs share the passes over the tile: about 1024 pixels each,
   // as far as every CTA of the launch has an SM of its own

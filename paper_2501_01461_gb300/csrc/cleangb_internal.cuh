@@ -231,9 +231,12 @@ cudaError_t select_prepare();  // kernel attributes
 // leave no component pending.
 cudaError_t launch_select(const PlanDev& d, int G, int smem, int parity, int flush, uint64_t limit_ns,
                           int force_timeout, cudaStream_t s);
-// One CTA per (image, tile) item.
+// G CTAs per (image, tile) item (G > 1: one cluster each); direct: tiles without
+// superblocks (SelDev::lq 0).
 cudaError_t launch_select_batch(const PlanDev* plans, const BatchItem* items, int n_items,
-                                int direct, int smem, int round, cudaStream_t s);
+                                int direct, int G, int smem, int round, uint64_t limit_ns,
+                                cudaStream_t s);
+bool select_cluster_fits(int direct, int G, int smem);
 
 // G CTAs per item (G = 1: independent CTAs; G > 1: one thread-block cluster
 // per item), each reading its image's plan state from `plans` (device
@@ -244,40 +247,6 @@ cudaError_t launch_minor_batch(const PlanDev* plans, const BatchItem* items, int
 // Largest cluster size <= want that can be scheduled for the batched kernel.
 int minor_batch_cluster(int want, int resident, int smem);
 
-// One tile of one image in the persistent batched minor loop: its launch
-// configuration (G CTAs with the grid exchange) and the body it takes.
-enum { kUnitResident = 0, kUnitTmem = 1, kUnitStreamed = 2, kUnitPair = 3 };
-struct BatchUnitItem {
-  MinorCfg cfg;
-  int32_t image;
-  int32_t tile;   // the tile, or for kUnitPair the pair (tiles 2 tile, 2 tile + 1)
-  int32_t kind;
-  int32_t ranks;  // CTAs of the unit: cfg.G, or 2 cfg.G for a pair
-};
-// CTAs of the persistent launch with `smem` bytes of dynamic shared memory
-// (one per SM; 0 if it cannot be resident).
-int minor_batch_persistent_grid(int smem);
-// One round of every item: units[w * grid + b] = (item, rank) of CTA b in
-// wave w, item -1 idle.  Cooperative launch.
-cudaError_t launch_minor_batch_persistent(const PlanDev* plans, const BatchUnitItem* items,
-                                          const int2* units, int n_waves, int grid, int smem,
-                                          const CUtensorMap* rmaps, const CUtensorMap* pmaps,
-                                          int round, cudaStream_t s);
-
-// Batched TMA pipeline: every image's residual and PSF box maps have boxes of
-// kBatchBoxW x kBatchBoxRows floats (chunks of 128 columns x 60 rows).
-constexpr int kBatchBoxW = 132;
-constexpr int kBatchBoxRows = 60;
-// Pipeline geometry for a batch group of G CTAs per tile whose CTAs hold at
-// most max_rows x max_w pixels (resident in shared memory or streamed);
-// false if the ring does not fit.
-bool minor_pipe_batch_geometry(MinorCfg& c, int G, int resident, int max_rows, int max_w);
-// Largest cluster size <= want (a power of two) the device can schedule for
-// the batched pipeline with `smem` bytes of dynamic shared memory (1 if none).
-int minor_pipe_batch_cluster(int want, int resident, int smem);
-cudaError_t launch_minor_pipe_batch(const PlanDev* plans, const BatchItem* items, int n_items,
-                                    const MinorCfg& c, const CUtensorMap* rmaps,
-                                    const CUtensorMap* pmaps, int round, cudaStream_t s);
 // Feedback for many images in one launch (plain loads, or TMA when maps is
 // non-NULL: one PSF tensor map per image in device memory, 64-byte aligned).
 cudaError_t launch_feedback_batch(const PlanDev* plans, const BatchImage* imgs, int n_images,
@@ -342,6 +311,8 @@ int minor_threads();
 PlanDev plan_device_state(const clean_plan_s* pl);
 bool plan_psf_tensor_map(const clean_plan_s* pl, CUtensorMap* out);
 int64_t plan_niter(const clean_plan_s* pl);
+// Dynamic shared memory of the plan's selection minor loop (0: not possible).
+int plan_select_smem(const clean_plan_s* pl);
 // FFT feedback of a plan on the state `d` (a batch job's copy of the plan's
 // device state, with its own control block and round phase).
 bool plan_uses_fft(const clean_plan_s* pl);

@@ -27,8 +27,8 @@
 //                        residual in tensor memory for the launch
 //   minor_pair_kernel    the pipeline with groups of 2G CTAs serving two tiles
 //                        alternately (grid groups, streamed rows, even T)
-//   minor_batch_kernel,  the same bodies over the (image, tile) items of a
-//   minor_pipe_batch_kernel  batch (one CTA or one cluster per item)
+//   minor_batch_kernel   the plain body over the (image, tile) items of a batch
+//                        (one CTA or one cluster per item)
 // Every variant gives the same bits.
 #include <algorithm>
 
@@ -677,10 +677,7 @@ constexpr int kTmemCols = 512;
 constexpr int kTmemChunks = 8;       // 4 warps per lane quarter x 8 chunks x 16 columns
 constexpr int kTmemChunkRows = 60;   // 15 warps x 4 slabs of one row
 
-// PERSIST: one unit of a persistent launch (the caller checks the plan's
-// status uniformly before; at the end the barriers are invalidated so the
-// next unit can initialise the same shared memory again).
-template <int SYNC, bool RES, bool TM = false, bool PERSIST = false>
+template <int SYNC, bool RES, bool TM = false>
 __device__ __forceinline__ void minor_pipe_body(const PlanDev& d, const MinorCfg& c, int parity,
                                                 const CUtensorMap* r_map,
                                                 const CUtensorMap* p_map, int t, int rank) {
@@ -714,7 +711,7 @@ __device__ __forceinline__ void minor_pipe_body(const PlanDev& d, const MinorCfg
   const uint64_t limit = (uint64_t)c.spin_limit_ns;
   const int WR = (W + 3) & ~3;              // resident slab row stride
 
-  if (!PERSIST && *(volatile int32_t*)&d.st->status != 0) return;  // uniform, see minor_kernel
+  if (*(volatile int32_t*)&d.st->status != 0) return;  // uniform, see minor_kernel
 
   // consumer geometry within a chunk: row slabs of 4-pixel groups (vector
   // path, CW = 32, 64 or 128) or single pixels, threads per row a power of two
@@ -735,9 +732,7 @@ __device__ __forceinline__ void minor_pipe_body(const PlanDev& d, const MinorCfg
   const bool tm_on = TM && n_tm > 0;
   if (tm_on && warp == 0) {
     ptx::tmem_alloc(&s_tmem, kTmemCols);
-    // a persistent CTA allocates again for its next unit: it keeps the permit
-    // (it owns its SM, so no other CTA waits for the columns)
-    if (!PERSIST) ptx::tmem_relinquish();
+    ptx::tmem_relinquish();
     ptx::tmem_fence_before_sync();
   }
 
@@ -1065,15 +1060,6 @@ __device__ __forceinline__ void minor_pipe_body(const PlanDev& d, const MinorCfg
     d.budget[t] = budget - k;
     d.gbar[t] = seq0 + (uint32_t)k;
   }
-  if (PERSIST) {
-    __syncthreads();
-    if (threadIdx.x == 0)
-      for (int i = 0; i < S; ++i) {
-        ptx::mbar_inval(&full_bar[i]);
-        ptx::mbar_inval(&empty_bar[i]);
-      }
-    __syncthreads();
-  }
 }
 
 template <int SYNC, bool RES, bool TM>
@@ -1197,8 +1183,7 @@ __device__ __forceinline__ uint64_t pair_poll(const PlanDev& d, const MinorCfg& 
   return abort ? 0ull : kk;
 }
 
-// PERSIST: one unit of the persistent batched launch (as in minor_pipe_body).
-template <bool TM, bool PERSIST = false>
+template <bool TM>
 __device__ __forceinline__ void minor_pair_body(const PlanDev& d, const MinorCfg& c, int parity,
                                                 const CUtensorMap* r_map,
                                                 const CUtensorMap* p_map, int pair, int q) {
@@ -1225,7 +1210,7 @@ __device__ __forceinline__ void minor_pair_body(const PlanDev& d, const MinorCfg
   const uint32_t p_box_bytes = (uint32_t)(BW * BH) * 4u;
   const uint64_t limit = (uint64_t)c.spin_limit_ns;
 
-  if (!PERSIST && *(volatile int32_t*)&d.st->status != 0) return;  // uniform, see minor_kernel
+  if (*(volatile int32_t*)&d.st->status != 0) return;  // uniform, see minor_kernel
 
   // per-tile state in named pairs (selected per step, no local arrays)
   const Piece pc0 = pair_piece(d, 2 * pair, q % G, q / G, G, BH, CW, TM && c.tmem);
@@ -1233,7 +1218,7 @@ __device__ __forceinline__ void minor_pair_body(const PlanDev& d, const MinorCfg
   const bool tm_on = TM && (pc0.n_tm > 0 || pc1.n_tm > 0);
   if (tm_on && warp == 0) {
     ptx::tmem_alloc(&s_tmem, kTmemCols);
-    if (!PERSIST) ptx::tmem_relinquish();  // a persistent CTA allocates again later
+    ptx::tmem_relinquish();
     ptx::tmem_fence_before_sync();
   }
 
@@ -1610,18 +1595,6 @@ __device__ __forceinline__ void minor_pair_body(const PlanDev& d, const MinorCfg
     d.budget[pc1.t] = budget1 - kx1;
     d.gbar[pc1.t] = seq01 + (uint32_t)kx1;
   }
-  if (PERSIST) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int i = 0; i < S; ++i) {
-        ptx::mbar_inval(&full_bar[i]);
-        ptx::mbar_inval(&empty_bar[i]);
-      }
-      ptx::mbar_inval(&key_bar[0]);
-      ptx::mbar_inval(&key_bar[1]);
-    }
-    __syncthreads();
-  }
 }
 
 template <bool TM>
@@ -1632,68 +1605,6 @@ __global__ void __launch_bounds__(kPipeThreads, 1)
   const int G2 = 2 * c.G;
   minor_pair_body<TM>(d, c, parity, &r_map, &p_map, (int)blockIdx.x / G2,
                       (int)blockIdx.x % G2);
-}
-
-// Batched pipeline launch: one CTA (kSyncNone) or one cluster of G CTAs per
-// (image, tile) item, each image's plan state in `plans` and its residual and
-// PSF box maps in rmaps / pmaps (global memory, indexed like `plans`).
-template <int SYNC, bool RES, bool TM>
-__global__ void __launch_bounds__(kPipeThreads, 1)
-    minor_pipe_batch_kernel(const PlanDev* __restrict__ plans,
-                            const BatchItem* __restrict__ items, const CUtensorMap* rmaps,
-                            const CUtensorMap* pmaps, MinorCfg c, int round) {
-  const BatchItem it = items[blockIdx.x / c.G];
-  const PlanDev d = plans[it.image];
-  const int rank = (SYNC == CLEAN_SYNC_CLUSTER) ? (int)cluster_rank() : 0;
-  minor_pipe_body<SYNC, RES, TM>(d, c, (round - d.round0) & 1, rmaps + it.image,
-                                 pmaps + it.image, it.tile, rank);
-}
-
-// Persistent batched minor loop: one CTA per SM, each working through its
-// column of a host-built schedule of waves.  units[w * gridDim.x + b] is the
-// (item, rank) that CTA b serves in wave w (item -1: idle).  An item is one
-// tile of one image with its own launch configuration; its G ranks sit in
-// one wave, so they run at the same time on distinct CTAs (the launch is
-// cooperative: every CTA is resident) and exchange their peaks through the
-// bounded grid exchange.  A CTA goes on to its next wave as soon as its unit
-// ends.  A CTA can only wait for the ranks of its own unit, and the ranks of
-// the earliest unfinished wave are all resident and at that unit, so the
-// schedule always progresses.  Each unit runs the pipelined body of the
-// single-plan and clustered kernels, so the results are bit for bit theirs.
-__global__ void __launch_bounds__(kPipeThreads, 1)
-    minor_batch_persistent_kernel(const PlanDev* __restrict__ plans,
-                                  const BatchUnitItem* __restrict__ items,
-                                  const int2* __restrict__ units, int n_waves,
-                                  const CUtensorMap* rmaps, const CUtensorMap* pmaps, int round) {
-  __shared__ int s_skip;
-  for (int w = 0; w < n_waves; ++w) {
-    const int2 u = units[(int64_t)w * gridDim.x + blockIdx.x];
-    if (u.x < 0) continue;  // the same for the whole CTA
-    const BatchUnitItem it = items[u.x];
-    const PlanDev d = plans[it.image];
-    if (threadIdx.x == 0) s_skip = *(volatile int32_t*)&d.st->status != 0;
-    __syncthreads();
-    const bool skip = s_skip != 0;
-    __syncthreads();
-    if (skip) continue;
-    const int parity = (round - d.round0) & 1;
-    const CUtensorMap* rm = rmaps + it.image;
-    const CUtensorMap* pm = pmaps + it.image;
-    switch (it.kind) {
-      case kUnitResident:
-        minor_pipe_body<CLEAN_SYNC_GRID, true, false, true>(d, it.cfg, parity, rm, pm, it.tile, u.y);
-        break;
-      case kUnitTmem:
-        minor_pipe_body<CLEAN_SYNC_GRID, false, true, true>(d, it.cfg, parity, rm, pm, it.tile, u.y);
-        break;
-      case kUnitPair:  // it.tile: the pair, tiles 2 it.tile and 2 it.tile + 1
-        minor_pair_body<true, true>(d, it.cfg, parity, rm, pm, it.tile, u.y);
-        break;
-      default:
-        minor_pipe_body<CLEAN_SYNC_GRID, false, false, true>(d, it.cfg, parity, rm, pm, it.tile, u.y);
-        break;
-    }
-  }
 }
 
 template <int SYNC, bool RES>
@@ -1749,136 +1660,6 @@ int minor_batch_cluster(int want, int resident, int smem) {
   }
   cudaGetLastError();
   return 1;
-}
-
-// ---- batched pipeline --------------------------------------------------------
-
-// tmem: the streamed variant that keeps each CTA's leading chunks in tensor
-// memory (every CTA owns its SM: the ring takes more than half of its
-// shared memory, so a later CTA starts there only after this one freed its
-// columns)
-const void* pipe_batch_fn(int G, int resident, int tmem) {
-  if (G > 1)
-    return resident ? (const void*)minor_pipe_batch_kernel<CLEAN_SYNC_CLUSTER, true, false>
-           : tmem   ? (const void*)minor_pipe_batch_kernel<CLEAN_SYNC_CLUSTER, false, true>
-                    : (const void*)minor_pipe_batch_kernel<CLEAN_SYNC_CLUSTER, false, false>;
-  return resident ? (const void*)minor_pipe_batch_kernel<kSyncNone, true, false>
-         : tmem   ? (const void*)minor_pipe_batch_kernel<kSyncNone, false, true>
-                  : (const void*)minor_pipe_batch_kernel<kSyncNone, false, false>;
-}
-
-bool minor_pipe_batch_geometry(MinorCfg& c, int G, int resident, int max_rows, int max_w) {
-  c = MinorCfg{};
-  c.G = G;
-  c.sync = G > 1 ? CLEAN_SYNC_CLUSTER : kSyncNone;
-  c.resident = resident;
-  c.spin_limit_ns = 2000000000ll;
-  c.chunk_w = 128;
-  c.box_w = kBatchBoxW;
-  c.chunk_h = kBatchBoxRows;
-  const int64_t box = (int64_t)((c.box_w * c.chunk_h + 31) & ~31) * 4;
-  const int64_t stage = (resident ? 1 : 2) * box;
-  c.res_floats = resident ? ((max_rows * ((max_w + 3) & ~3) + 31) & ~31) : 0;
-  const int64_t budget = 200 * 1024 - (int64_t)c.res_floats * 4;
-  c.stages = (int)std::min<int64_t>(kPipeMaxStages, budget / stage);
-  if (c.stages < 2) return false;
-  c.smem = (int)((int64_t)c.res_floats * 4 + c.stages * stage);
-  c.threads = kPipeThreads;
-  c.pipe = 1;
-  c.tmem = (!resident && c.smem > 114 * 1024) ? 1 : 0;
-  return true;
-}
-
-int minor_pipe_batch_cluster(int want, int resident, int smem) {
-  for (int G = std::min(16, std::max(1, want)); G > 1; G /= 2) {
-    const void* fn = pipe_batch_fn(G, resident, 0);
-    if (allow_max_smem(fn) != cudaSuccess) break;
-    if (G > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-                     cudaSuccess)
-      continue;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(G, 1, 1);
-    cfg.blockDim = dim3(kPipeThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = G;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n >= 1) return G;
-  }
-  cudaGetLastError();
-  return 1;
-}
-
-cudaError_t launch_minor_pipe_batch(const PlanDev* plans, const BatchItem* items, int n_items,
-                                    const MinorCfg& c, const CUtensorMap* rmaps,
-                                    const CUtensorMap* pmaps, int round, cudaStream_t s) {
-  if (n_items <= 0) return cudaSuccess;
-  const void* fn = pipe_batch_fn(c.G, c.resident, c.tmem);
-  cudaError_t e = allow_max_smem(fn);
-  if (e != cudaSuccess) return e;
-  if (c.G > 8) {
-    e = cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-    if (e != cudaSuccess) return e;
-  }
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)(n_items * c.G), 1, 1);
-  cfg.blockDim = dim3(kPipeThreads, 1, 1);
-  cfg.dynamicSmemBytes = c.smem;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = c.G;
-  at[0].val.clusterDim.y = 1;
-  at[0].val.clusterDim.z = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = c.G > 1 ? 1 : 0;
-  MinorCfg cc = c;
-  void* args[] = {const_cast<PlanDev**>(&plans), const_cast<BatchItem**>(&items),
-                  const_cast<CUtensorMap**>(&rmaps), const_cast<CUtensorMap**>(&pmaps), &cc,
-                  &round};
-  return cudaLaunchKernelExC(&cfg, fn, args);
-}
-
-int minor_batch_persistent_grid(int smem) {
-  const void* fn = (const void*)minor_batch_persistent_kernel;
-  int dev = 0, sms = 0, per_sm = 0;
-  if (allow_max_smem(fn) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kPipeThreads, smem) !=
-          cudaSuccess) {
-    cudaGetLastError();
-    return 0;
-  }
-  return per_sm >= 1 ? sms : 0;  // one CTA per SM (the tensor-memory units own their SM)
-}
-
-cudaError_t launch_minor_batch_persistent(const PlanDev* plans, const BatchUnitItem* items,
-                                          const int2* units, int n_waves, int grid, int smem,
-                                          const CUtensorMap* rmaps, const CUtensorMap* pmaps,
-                                          int round, cudaStream_t s) {
-  if (n_waves <= 0 || grid <= 0) return cudaSuccess;
-  const void* fn = (const void*)minor_batch_persistent_kernel;
-  cudaError_t e = allow_max_smem(fn);
-  if (e != cudaSuccess) return e;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid, 1, 1);
-  cfg.blockDim = dim3(kPipeThreads, 1, 1);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeCooperative;
-  at[0].val.cooperative = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  void* args[] = {const_cast<PlanDev**>(&plans), const_cast<BatchUnitItem**>(&items),
-                  const_cast<int2**>(&units), &n_waves, const_cast<CUtensorMap**>(&rmaps),
-                  const_cast<CUtensorMap**>(&pmaps), &round};
-  return cudaLaunchKernelExC(&cfg, fn, args);
 }
 
 cudaError_t launch_minor_batch(const PlanDev* plans, const BatchItem* items, int n_items, int G,

@@ -1131,14 +1131,15 @@ __global__ void __launch_bounds__(kThreads, 1)
                       (int)blockIdx.x % G);
 }
 
-// One CTA per (image, tile) item: no CTA waits on another.
+// G CTAs per (image, tile) item; with G > 1 they form one cluster, so they run
+// at the same time and may wait for each other.
 template <bool DIRECT>
 __global__ void __launch_bounds__(kThreads, 1)
     select_batch_kernel(const PlanDev* __restrict__ plans, const BatchItem* __restrict__ items,
-                        int round) {
-  const BatchItem it = items[blockIdx.x];
+                        int G, int round, uint64_t limit_ns) {
+  const BatchItem it = items[blockIdx.x / G];
   const PlanDev d = plans[it.image];
-  select_body<DIRECT>(d, 1, (round - d.round0) & 1, 0, 0, 0, it.tile, 0);
+  select_body<DIRECT>(d, G, (round - d.round0) & 1, 0, limit_ns, 0, it.tile, blockIdx.x % G);
 }
 
 // ---- the PSF's ranges (once per PSF) -------------------------------------------
@@ -1312,14 +1313,47 @@ cudaError_t launch_select(const PlanDev& d, int G, int smem, int parity, int flu
       args);
 }
 
+namespace {
+void batch_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int n_items, int G, int smem) {
+  *cfg = cudaLaunchConfig_t{};
+  cfg->gridDim = dim3((unsigned)(n_items * G), 1, 1);
+  cfg->blockDim = dim3(kThreads, 1, 1);
+  cfg->dynamicSmemBytes = smem;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = G;
+  at->val.clusterDim.y = 1;
+  at->val.clusterDim.z = 1;
+  cfg->attrs = at;
+  cfg->numAttrs = G > 1 ? 1 : 0;
+}
+const void* batch_fn(int direct) {
+  return direct ? (const void*)select_batch_kernel<true> : (const void*)select_batch_kernel<false>;
+}
+}  // namespace
+
+bool select_cluster_fits(int direct, int G, int smem) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at;
+  batch_config(&cfg, &at, 1, G, smem);
+  int n = 0;
+  if (cudaOccupancyMaxActiveClusters(&n, batch_fn(direct), &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return n >= 1;
+}
+
 cudaError_t launch_select_batch(const PlanDev* plans, const BatchItem* items, int n_items,
-                                int direct, int smem, int round, cudaStream_t s) {
+                                int direct, int G, int smem, int round, uint64_t limit_ns,
+                                cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
-  if (direct)
-    select_batch_kernel<true><<<n_items, kThreads, smem, s>>>(plans, items, round);
-  else
-    select_batch_kernel<false><<<n_items, kThreads, smem, s>>>(plans, items, round);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute at;
+  batch_config(&cfg, &at, n_items, G, smem);
+  cfg.stream = s;
+  void* args[] = {const_cast<PlanDev**>(&plans), const_cast<BatchItem**>(&items), &G, &round,
+                  &limit_ns};
+  return cudaLaunchKernelExC(&cfg, batch_fn(direct), args);
 }
 
 }  // namespace cleangb
