@@ -95,3 +95,25 @@ def test_step_leaves_nothing_pending():
         r, _, _ = p.get()
         o = oracle.clean_f32(dirty, psf, 0.1, 200, 0.0, (2, 2), 20)
         assert np.array_equal(r.cpu().numpy().view(np.uint32), o.residual.view(np.uint32))
+
+
+@pytest.mark.parametrize("ny,nx,dense", [(64, 64, 0), (65, 200, 0), (31, 17, 1), (130, 70, 1)])
+def test_restore_of_sparse_and_dense_models(ny, nx, dense):
+    """Output blocks at and past their edges; a model with few and with all
+    pixels non-zero (several lists a block), against the float64 restore."""
+    import torch
+    rng = np.random.default_rng(ny)
+    psf = np.zeros((2 * ny, 2 * nx), np.float32)
+    psf[ny, nx] = 1.0
+    dirty = synth.random_image(ny, nx, rng)
+    niter = ny * nx if dense else 20
+    with cg.Plan(torch.from_numpy(psf).cuda(), ny, nx, gain=1.0, niter=niter) as p:
+        p.run(torch.from_numpy(dirty).cuda())
+        r, m, _ = p.get()
+        out = p.restore(9.5, 7.25, 0.6).cpu().numpy()
+    r, m = r.cpu().numpy(), m.cpu().numpy()
+    assert (m != 0).sum() == niter
+    want = oracle.restore(m, r, 9.5, 7.25, float(np.float32(0.6)))
+    # each of up to 41^2 terms and their sum in float32, beam values to 1e-6
+    bound = 41 * 41 * 2.0 ** -24 * np.abs(m).max() * 100 + 2e-6 * np.abs(m).max() * 100
+    assert np.abs(out - want).max() <= bound
