@@ -12,10 +12,10 @@
 // they would have in a loop that subtracts each at once.
 //
 // Each CTA owns a kRows x kCols block of one tile; every thread keeps its
-// kRowsPerWarp x kColsPerLane pixels in registers for the whole component
-// list, so the residual is read and written once per round.  The CTA also
-// reduces its pixels' peak key (largest |R|, lowest index) into the tile's
-// next-round peak with a 64-bit atomic max.
+// pixels in registers for the whole component list, so the residual is read
+// and written once per round.  The CTA also reduces its pixels' peak key
+// (largest |R|, lowest index) into the tile's next-round peak with a 64-bit
+// atomic max.
 //
 // The last CTA to finish closes the round: it appends the round's
 // components to the list (round-major, then tile, then iteration), records
@@ -33,18 +33,24 @@ namespace cleangb {
 
 namespace {
 
-constexpr int kWarps = 8;
+// Plain loads: a block is 16 rows x 64 columns, a warp 8 x 32 of them with a
+// column a lane, so a window's row is 32 neighbours whatever its alignment, and
+// kAhead components' windows are on their way together.  Bound by L2 latency
+// on the images that come here (PSF rows off 16 bytes, or narrower than the
+// TMA box).  The block is small for the sake of small images: 301 x 277 in
+// six tiles, 250 components a round, 126 blocks: about 30 us a round, 203 with
+// 64 x 64 blocks and one component at a time.
+constexpr int kWarps = 4;
 constexpr int kThreads = kWarps * 32;
-constexpr int kRowsPerWarp = 8;
-constexpr int kColsPerLane = 2;
-constexpr int kRows = kWarps * kRowsPerWarp;  // 64
-constexpr int kCols = 32 * kColsPerLane;      // 64
-constexpr int kChunk = 512;                   // components staged at once
+constexpr int kUnitRows = 8;                  // rows a warp holds
+constexpr int kRows = 16, kCols = 64;
+constexpr int kAhead = 4;
+constexpr int kChunk = 256;                   // components staged at once
 
 struct __align__(16) Comp4 {
-  int32_t y, x;
+  int32_t y, x;    // PSF row and column of the block's first pixel
   float f;
-  int32_t pad;
+  int32_t full;    // the block's pixels' window lies inside the PSF
 };
 
 // Sum of the round's component counts over all tiles (0: the round changed
@@ -91,47 +97,66 @@ __device__ __forceinline__ void feedback_body(const PlanDev& d, int parity, int 
     const int own0 = d.rapplied[t], n_own = d.rcount[t] - own0;
     const int n_list = n_own + s_pre[d.T];
 
-    float r[kRowsPerWarp][kColsPerLane];
-    bool in[kRowsPerWarp][kColsPerLane];
+    const int by1 = min(rc.y1, by0 + kRows), bx1 = min(rc.x1, bx0 + kCols);
+    const int y0 = by0 + (warp >> 1) * kUnitRows, x = bx0 + (warp & 1) * 32 + lane;
+    const int rows = x < bx1 ? max(0, min(kUnitRows, by1 - y0)) : 0;
+    // pixels that do not exist read the window at the block's edge
+    const int dy = min(y0, by1 - 1) - by0, dx = min(x, bx1 - 1) - bx0;
+    int step[kUnitRows];
 #pragma unroll
-    for (int i = 0; i < kRowsPerWarp; ++i)
+    for (int i = 0; i < kUnitRows; ++i) step[i] = min(i, by1 - 1 - by0 - dy) * d.pnx;
+    float r[kUnitRows];
 #pragma unroll
-      for (int j = 0; j < kColsPerLane; ++j) {
-        const int y = by0 + warp * kRowsPerWarp + i;
-        const int x = bx0 + lane + 32 * j;
-        in[i][j] = y < rc.y1 && x < rc.x1;
-        r[i][j] = in[i][j] ? d.R[(int64_t)y * d.nx + x] : 0.f;
-      }
+    for (int i = 0; i < kUnitRows; ++i)
+      r[i] = i < rows ? d.R[(int64_t)(y0 + i) * d.nx + x] : 0.f;
 
-    const int y_first = by0 + warp * kRowsPerWarp;
-    const int x_first = bx0 + lane;
     for (int base = 0; base < n_list; base += kChunk) {
       const int n = min(kChunk, n_list - base);
       __syncthreads();
       for (int jj = threadIdx.x; jj < n; jj += kThreads) {
         const clean_component cc = list_component(d, t, base + jj, own0, n_own, s_pre);
         Comp4 c4;
-        c4.y = cc.y;
-        c4.x = cc.x;
+        c4.y = by0 - cc.y + d.cy;
+        c4.x = bx0 - cc.x + d.cx;
         c4.f = cc.flux;
-        c4.pad = 0;
+        c4.full = c4.y >= 0 && c4.y + (by1 - by0) <= d.pny && c4.x >= 0 &&
+                  c4.x + (bx1 - bx0) <= d.pnx;
         s_comp[jj] = c4;
       }
       __syncthreads();
-      for (int jj = 0; jj < n; ++jj) {
-        const Comp4 c4 = s_comp[jj];
-        const int sy0 = y_first - c4.y + d.cy;
-        const int sx0 = x_first - c4.x + d.cx;
+      for (int j0 = 0; j0 < n; j0 += kAhead) {
+        Comp4 c[kAhead];
+        int full = 1;
 #pragma unroll
-        for (int i = 0; i < kRowsPerWarp; ++i) {
-          const int sy = sy0 + i;
-          const bool yin = (unsigned)sy < (unsigned)d.pny;
+        for (int u = 0; u < kAhead; ++u) {
+          c[u] = s_comp[min(j0 + u, n - 1)];
+          full &= c[u].full;
+        }
+        if (full) {
+          float p[kAhead][kUnitRows];
 #pragma unroll
-          for (int j = 0; j < kColsPerLane; ++j) {
-            const int sx = sx0 + 32 * j;
-            if (in[i][j] && yin && (unsigned)sx < (unsigned)d.pnx) {
-              const float p = __ldg(d.P + (int64_t)sy * d.pnx + sx);
-              r[i][j] = __fsub_rn(r[i][j], __fmul_rn(c4.f, p));
+          for (int u = 0; u < kAhead; ++u) {
+            const float* w = d.P + ((int64_t)(c[u].y + dy) * d.pnx + c[u].x + dx);
+#pragma unroll
+            for (int i = 0; i < kUnitRows; ++i) p[u][i] = ptx::ld_nc(w + step[i]);
+          }
+#pragma unroll
+          for (int u = 0; u < kAhead; ++u)
+            if (j0 + u < n) {
+#pragma unroll
+              for (int i = 0; i < kUnitRows; ++i) r[i] = __fsub_rn(r[i], __fmul_rn(c[u].f, p[u][i]));
+            }
+        } else {
+          // windows partly off the PSF array: those pixels stay unchanged
+#pragma unroll 1
+          for (int j = j0; j < min(j0 + kAhead, n); ++j) {
+            const Comp4 e = s_comp[j];
+            const int sx = e.x + dx;
+#pragma unroll
+            for (int i = 0; i < kUnitRows; ++i) {
+              const int sy = e.y + y0 - by0 + i;
+              if (i < rows && (unsigned)sy < (unsigned)d.pny && (unsigned)sx < (unsigned)d.pnx)
+                r[i] = __fsub_rn(r[i], __fmul_rn(e.f, __ldg(d.P + (int64_t)sy * d.pnx + sx)));
             }
           }
         }
@@ -142,21 +167,17 @@ __device__ __forceinline__ void feedback_body(const PlanDev& d, int parity, int 
     float best_a = -1.f, best_v = 0.f;
     int best_i = 0x7fffffff;
 #pragma unroll
-    for (int i = 0; i < kRowsPerWarp; ++i)
-#pragma unroll
-      for (int j = 0; j < kColsPerLane; ++j) {
-        if (!in[i][j]) continue;
-        const int y = by0 + warp * kRowsPerWarp + i;
-        const int x = bx0 + lane + 32 * j;
-        const int gi = y * d.nx + x;
-        if (n_list > 0) d.R[(int64_t)gi] = r[i][j];
-        const float a = fabsf(r[i][j]);
-        if (a > best_a || (a == best_a && gi < best_i)) {
-          best_a = a;
-          best_i = gi;
-          best_v = r[i][j];
-        }
+    for (int i = 0; i < kUnitRows; ++i) {
+      if (i >= rows) continue;
+      const int gi = (y0 + i) * d.nx + x;
+      if (n_list > 0) d.R[(int64_t)gi] = r[i];
+      const float a = fabsf(r[i]);
+      if (a > best_a) {  // rows ascend: the first keeps a tie
+        best_a = a;
+        best_i = gi;
+        best_v = r[i];
       }
+    }
     uint64_t k = best_a >= 0.f ? make_key(best_v, best_i) : 0ull;
     k = warp_max_key(k);
     if (lane == 0) s_warp[warp] = k;

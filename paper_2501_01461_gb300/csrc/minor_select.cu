@@ -166,15 +166,8 @@ __device__ __forceinline__ Geo make_geo(const PlanDev& d, int t) {
   return g;
 }
 
-// A load of the PSF that stays where it is written: the compiler would move
-// plain loads down to their uses, one at a time, to save registers.
-__device__ __forceinline__ float ld_psf(const float* p) {
-  float v;
-  asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
-  return v;
-}
-
-__device__ __forceinline__ float ld_res(const float* p) {  // likewise, of the residual
+// A load of the residual that stays where it is written (see ptx::ld_nc).
+__device__ __forceinline__ float ld_res(const float* p) {
   float v;
   asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
   return v;
@@ -204,8 +197,8 @@ __device__ __forceinline__ void less_pending(const PlanDev& d, float (&r)[2],
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int o = s.comp[j0 + u].w;
-        p[u][0] = ld_psf(P0 + o);
-        p[u][1] = ld_psf(P1 + o);
+        p[u][0] = ptx::ld_nc(P0 + o);
+        p[u][1] = ptx::ld_nc(P1 + o);
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -285,7 +278,7 @@ __device__ __forceinline__ void tile_pass(const PlanDev& d, const Geo& g, int ra
           for (int c = 0; c < U; ++c) {
             const float* Pp = Pb + s.comp[j + c].w;
 #pragma unroll
-            for (int i = 0; i < kUnitRows; ++i) p[c][i] = ld_psf(Pp + step[i]);
+            for (int i = 0; i < kUnitRows; ++i) p[c][i] = ptx::ld_nc(Pp + step[i]);
           }
 #pragma unroll
           for (int c = 0; c < U; ++c) {
@@ -846,7 +839,7 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
       ok[i] = i * kThreads < ncand;
       if (!ok[i]) continue;
       if (d.sel.inside)
-        pv[i] = ld_psf(d.P + (off + at[i]));
+        pv[i] = ptx::ld_nc(d.P + (off + at[i]));
       else
         ok[i] = psf_at(d, (int)(pos[i] >> 15) - pyl + d.cy, (int)(pos[i] & 0x7fffu) - pxl + d.cx,
                        &pv[i]);
