@@ -57,14 +57,19 @@ __device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t b
       : "memory");
 }
 
-int fft_sm_count() {
-  int dev = 0, n = 0;
+// CTAs of a persistent launch: as many as are resident at once.  One a SM left
+// short transforms with few warps in flight (192 threads at length 3000, a
+// 1500^2 image: two rounds took 1.11 ms, now 0.90; at length 8192, where one CTA
+// fills the SM, both 1.80).
+int fft_resident_ctas(const void* fn, int threads, size_t smem) {
+  int dev = 0, sms = 0, per = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, fn, threads, smem) != cudaSuccess) {
     cudaGetLastError();
     return 1;
   }
-  return std::max(n, 1);
+  return std::max(sms, 1) * std::max(per, 1);
 }
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
@@ -558,7 +563,7 @@ __global__ void __launch_bounds__(kCompThreads)
   if (threadIdx.x == 0) comps[0] = make_int4(n, s_rows, 0, 0);
 }
 
-// Columns k = blockIdx.x, blockIdx.x + gridDim.x, ... (one CTA per SM):
+// Columns k = blockIdx.x, blockIdx.x + gridDim.x, ... (every resident CTA):
 // the components' x-axis DFT at k placed on their rows, forward FFT along y,
 // times the kernel spectrum, inverse FFT along y; rows 0 .. ny - 1 to Y
 // (pair-major, below).  The components of one row are summed in list order (their
@@ -730,8 +735,8 @@ struct PairOut {  // R <- R0 - S for the pair's image columns; (R q0, R q1) back
   }
 };
 
-// Pairs of rows b = blockIdx.x, blockIdx.x + gridDim.x, ... (one CTA per
-// SM), rows q0 = 2b and q1 = 2b + 1: their x-axis spectra (one contiguous
+// Pairs of rows b = blockIdx.x, blockIdx.x + gridDim.x, ... (every resident
+// CTA), rows q0 = 2b and q1 = 2b + 1: their x-axis spectra (one contiguous
 // run of Y) extended to length Lx and combined as Z = Y_q0 + i Y_q1; the
 // inverse FFT gives row q0 in the real and row q1 in the imaginary part.
 // R <- R0 - S, R0 <- R on columns 0 .. nx - 1; each tile's peak of these
@@ -1008,11 +1013,12 @@ cudaError_t fft_feedback_round(const PlanDev& d, const FftAxis& ay, const FftAxi
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int ncols = ax.L / 2 + 1;
-  const int grid = std::min(ncols, fft_sm_count());
   // the spectrum column, the transform, then the radix-16 path's component
   // rows or the mixed-radix path's second buffer
   const size_t cs = sizeof(float2) * (size_t)ay.L + fft_smem_bytes(ay.L) +
                     (ay.p2 ? sizeof(float2) * (size_t)d.ny : fft_smem_bytes(ay.L));
+  const void* cfn = ay.p2 ? (const void*)fft_cols_kernel<true> : (const void*)fft_cols_kernel<false>;
+  const int grid = std::min(ncols, fft_resident_ctas(cfn, ay.nthr, cs));
   if (ay.p2)
     fft_cols_kernel<true><<<grid, ay.nthr, cs, s>>>(d, ay, ax.L, comps, lead, twx, twy, Kspec, Y,
                                                     kFftWaitNs);
@@ -1022,11 +1028,12 @@ cudaError_t fft_feedback_round(const PlanDev& d, const FftAxis& ay, const FftAxi
   e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const int npairs = (d.ny + 1) / 2;
-  const int rgrid = std::min(npairs, fft_sm_count());
   size_t smem = sizeof(float2) * 2 * (size_t)((ncols + 1) & ~1) +
                 sizeof(float) * 2 * (size_t)((d.nx + 3) & ~3) + fft_smem_bytes(ax.L) +
                 sizeof(int32_t) * (2 * (size_t)d.T + 1);
   if (ax.p2) {
+    const int rgrid =
+        std::min(npairs, fft_resident_ctas((const void*)fft_rows_kernel<true>, ax.nthr, smem));
     fft_rows_kernel<true><<<rgrid, ax.nthr, smem, s>>>(d, ax, twx, Y, R0, parity, kFftWaitNs, 0);
     return cudaGetLastError();
   }
@@ -1047,6 +1054,8 @@ cudaError_t fft_feedback_round(const PlanDev& d, const FftAxis& ay, const FftAxi
     }
     cudaGetLastError();
   }
+  const int rgrid =
+      std::min(npairs, fft_resident_ctas((const void*)fft_rows_kernel<false>, ax.nthr, smem));
   fft_rows_kernel<false><<<rgrid, ax.nthr, smem, s>>>(d, ax, twx, Y, R0, parity, kFftWaitNs,
                                                       scratch);
   return cudaGetLastError();
