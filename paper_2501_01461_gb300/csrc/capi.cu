@@ -52,8 +52,8 @@ struct clean_plan_s {
   int sel_G = 1;               // CTAs per tile
   int sel_smem = 0;
   float2* sel_boxes = nullptr; // work area of the PSF tables
-  float2* sel_h8 = nullptr;
-  float2* sel_hb = nullptr;
+  uint32_t* sel_h8 = nullptr;
+  uint32_t* sel_hb = nullptr;
   uint32_t* sel_lobe = nullptr;
   int max_rows = 0, max_w = 0;  // largest CTA slab of the minor loop
   float* psf_own = nullptr;
@@ -826,7 +826,7 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
     req.push_back({(void**)&pl->d.sel.ctl, sel_z.ctl});
     req.push_back({(void**)&pl->sel_boxes, sel_z.boxes});
     req.push_back({(void**)&pl->sel_h8, sel_z.h8});
-    req.push_back({(void**)&pl->sel_hb, sel_z.hb});
+    if (sel_z.hb) req.push_back({(void**)&pl->sel_hb, sel_z.hb});
     req.push_back({(void**)&pl->sel_lobe, sel_z.lobe});
   }
   size_t total = 0;

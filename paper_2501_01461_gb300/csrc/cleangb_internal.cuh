@@ -96,14 +96,14 @@ struct SelCtl {
 struct SelDev {
   float2* u;            // [T][cell_stride] bounds of R and -R per 8 x 8 cell
   uint2* masks;         // [T][cell_stride] the cells' pixels that are candidates
-  const float2* h8;     // PSF range over the windows a cell can meet
-  const float2* hb;     // the same for a superblock of (1 << lq)^2 cells
+  const uint32_t* h8;   // PSF range over the windows a cell can meet, by the
+                        // cells from the peak's to it (two bf16, see pack_rises)
+  const uint32_t* hb;   // the same for a superblock of (1 << lq)^2 cells, by its first
   const uint32_t* lobe; // exact ranges of the 8 x 8 cells around a peak
   SelCtl* ctl;          // [T]
   int64_t cell_stride;  // cells of the largest tile (rows of `pitch`)
   int32_t lq, pitch;
-  int32_t oy8, ox8, w8; // h8: entry of offset box 0, row length
-  int32_t oyb, oxb, wb; // hb likewise
+  int32_t oy8, ox8, w8; // h8 and hb: entry of offset 0, row length
   int32_t inside;       // the PSF array holds every offset between two pixels of a tile
 };
 struct SelSizes {
@@ -224,7 +224,7 @@ cudaError_t minor_prepare(const MinorCfg& c);  // sets function attributes
 // too large for the packed positions.
 bool select_geometry(SelDev* g, int ny, int nx, int ty, int tx, SelSizes* z);
 // The PSF's range tables (after every PSF change); boxes: work area.
-cudaError_t select_build_psf(const PlanDev& d, float2* boxes, float2* h8, float2* hb,
+cudaError_t select_build_psf(const PlanDev& d, float2* boxes, uint32_t* h8, uint32_t* hb,
                              uint32_t* lobe, cudaStream_t s);
 cudaError_t select_prepare();  // kernel attributes
 // One round's minor loops, G CTAs a tile (G > 1: a cooperative launch); flush:

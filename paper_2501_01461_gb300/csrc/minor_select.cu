@@ -34,8 +34,13 @@
 //
 // Bounds come in two levels so that an iteration touches few of them: a
 // superblock of Q x Q cells (Q a power of two, at most kMaxSb superblocks a
-// tile) has one offset added to all its cells; only the 4 x 4 superblocks
-// around the peak, where the PSF varies fast, raise their cells one by one.
+// tile) has one offset added to all its cells; only the superblocks around the
+// peak, where the PSF varies fast, raise their cells one by one.  The offsets'
+// table has an entry for every cell the superblock can lie away from the peak,
+// not only for every superblock: windows of (Q + 1)^2 boxes, not (2 Q)^2, rise
+// less, and the cells one by one are those of 2 x 2 superblocks (3 x 3 of
+// 4 x 4 cells), not of 4 x 4.  It does not fit shared memory and need not: its
+// L2 round trip runs beside the candidates'.
 //
 // What bounds it: an iteration is a chain of about 1400 cycles (0.7 us: decode,
 // one L2 round trip of the candidates' PSF gather at one L1 tag a candidate,
@@ -128,7 +133,7 @@ struct SelShared {
   unsigned long long key;     // the pass's peak key (this CTA's part)
   long long k_cmd;            // the group's command: components so far, finished
   int done_cmd, abort;
-  // followed by the superblocks' PSF ranges
+  // followed by the cells' PSF ranges (SelDev::h8) in tiles without superblocks
 };
 
 // The kernel's shared memory.  Every function names it itself, so that the
@@ -171,6 +176,15 @@ __device__ __forceinline__ float ld_res(const float* p) {
   float v;
   asm volatile("ld.global.cg.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
   return v;
+}
+
+__device__ __forceinline__ float2 ld_cell(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ uint32_t ld_range(const uint32_t* p) {
+  return __float_as_uint(ptx::ld_nc(reinterpret_cast<const float*>(p)));
 }
 
 // PSF value at an index of the array, and whether the index lies inside.
@@ -642,10 +656,9 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
                                                  uint32_t abs0, uint32_t lo0, int64_t k0,
                                                  int64_t kmax, float level, bool* done) {
   SelShared& s = shared_state();
-  uint2* const hbt = reinterpret_cast<uint2*>(sel_smem + sizeof(SelShared));
-  const uint32_t* const hbd = reinterpret_cast<const uint32_t*>(hbt);  // DIRECT: bf16 pairs
+  uint32_t* const h8s = reinterpret_cast<uint32_t*>(sel_smem + sizeof(SelShared));  // DIRECT
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int ns = g.nsy * g.nsx, nc = g.ncy * g.pitch, lq = g.lq, lB = 3 + lq, Q = 1 << lq;
+  const int ns = g.nsy * g.nsx, nc = g.ncy * g.pitch, lq = g.lq, Q = 1 << lq;
   const float stop = fmaxf(d.thr, level);  // threshold, flux trigger
   *done = false;
   if (k0 >= kmax || (abs0 | lo0) == 0u || !(__uint_as_float(abs0) > stop)) {
@@ -662,11 +675,11 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
   if (tid == 0) s.n_cells = s.n_sbs = s.n_cand = 0;
   for (int i = tid; i < 64 * 64 / 4; i += kThreads)
     reinterpret_cast<uint4*>(s.lobe)[i] = __ldg(reinterpret_cast<const uint4*>(d.sel.lobe) + i);
-  {
-    const int n = (2 * d.sel.oyb + 1) * d.sel.wb, n8 = DIRECT ? (n + 1) / 2 : n;  // 8-byte words
+  if (DIRECT) {
+    const int n8 = ((2 * d.sel.oy8 + 1) * d.sel.w8 + 1) / 2;  // 8-byte words
 #pragma unroll 2
     for (int i = tid; i < n8; i += kThreads)
-      hbt[i] = __ldg(reinterpret_cast<const uint2*>(d.sel.hb) + i);
+      reinterpret_cast<uint2*>(h8s)[i] = __ldg(reinterpret_cast<const uint2*>(d.sel.h8) + i);
   }
   __syncthreads();
   if (room > 1) {
@@ -737,26 +750,27 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
   // ... its superblocks' (DIRECT: cells') places in the table of PSF ranges, and
   // their offsets (bounds; shared memory has the offsets too) ...
   constexpr int kOwn = DIRECT ? kDirPer : kSbPer;
-  int hbi[kOwn];
+  int hbi[kOwn], sby[DIRECT ? 1 : kOwn], sbx[DIRECT ? 1 : kOwn];
   float2 acc[kOwn];
 #pragma unroll
   for (int i = 0; i < kOwn; ++i) {
     const int b = tid + i * kThreads, y = b < ns ? b / g.nsx : 0, x = b < ns ? b - y * g.nsx : 0;
-    hbi[i] = y * d.sel.wb + x;
+    hbi[i] = ((y << lq) + d.sel.oy8) * d.sel.w8 + (x << lq) + d.sel.ox8;
+    if (!DIRECT) {
+      sby[i] = y;
+      sbx[i] = x;
+    }
     acc[i] = make_float2(0.f, 0.f);
     if (DIRECT)
       acc[i] = b < ns ? __ldcg(&g.u[(int64_t)y * g.pitch + x]) : make_float2(-INFINITY, -INFINITY);
   }
-  // ... and its cell among the 4 x 4 superblocks around the peak, nL lanes a
+  // ... and its cell among the nb x nb superblocks around the peak that its
+  // 8 x 8 cells reach (superblocks have 4 x 4 cells at least), nL lanes a
   // superblock (for larger superblocks, its first cell)
+  const int nb = lq >= 3 ? 2 : 3;
   const int nlw = min(2 * lq, 5), nL = 1 << nlw;
-  const int nq0 = tid >> nlw, nc0 = tid & (nL - 1);
-
-  // the model, summed in list order by one thread: a pixel's sum stays in a
-  // register while its components follow one another, and a new pixel's value
-  // is on its way until the next component
-  float* mp = nullptr;
-  float mval = 0.f, mflux = 0.f;
+  const int nq = tid >> nlw, nc0 = tid & (nL - 1);
+  const bool near_warp = !DIRECT && (nq & -(32 >> nlw)) < nb * nb;  // (one for the warp)
 
   uint32_t wabs = abs0, wlo = lo0;
   int n = 0, buf = 0, spent = 0;
@@ -775,26 +789,7 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
     const int pyl = (int)(p >> 15), pxl = (int)(p & 0x7fffu);
     const float f = __fmul_rn(d.gain, __uint_as_float(wabs | (wlo << 31)));  // first equation
     const int off = (d.cy - pyl) * d.pnx + d.cx - pxl;
-    // (three warps share the record keeping)
-    if (tid == kThreads - 96) s.comp[n] = make_int4(pyl, pxl, __float_as_int(f), off);
-    if (tid == kThreads - 64) {
-      clean_component cc;
-      cc.y = g.rc.y0 + pyl;
-      cc.x = g.rc.x0 + pxl;
-      cc.flux = f;
-      cc.tile = t;
-      d.rcomps[(int64_t)t * d.cap_round + k0 + n] = cc;
-    }
-    if (tid == kThreads - 32) {
-      float* q = d.model + (int64_t)(g.rc.y0 + pyl) * d.nx + g.rc.x0 + pxl;
-      if (mp) mval = __fadd_rn(mval, mflux);
-      if (q != mp) {
-        if (mp) __stcg(mp, mval);
-        mp = q;
-        mval = __ldcg(q);
-      }
-      mflux = f;
-    }
+    if (tid == kThreads - 32) s.comp[n] = make_int4(pyl, pxl, __float_as_int(f), off);
     ++n;
     // (values that could overflow go one component at a time, as the plain
     // loop sees them)
@@ -805,30 +800,51 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
     }
     E = __fmaf_ru(reach, 0x1p-22f, E);
     // ---- the loads: the PSF ranges (the largest rise of R and of -R for
-    // f = 1; an entry below 0 marks the 4 x 4 superblocks whose windows can hold
-    // the peak's surroundings), then the candidates' PSF values ----
-    const int cyl = (pyl + (1 << lB) - 1) >> lB, cxl = (pxl + (1 << lB) - 1) >> lB;
-    const int hb0 = (d.sel.oyb - cyl) * d.sel.wb + d.sel.oxb - cxl;
+    // f = 1), then the candidates' PSF values ----
+    const int cyl = (pyl + 7) >> 3, cxl = (pxl + 7) >> 3, h0 = -(cyl * d.sel.w8 + cxl);
     // the first of the 8 x 8 cells around the peak, and their ranges for the
     // peak's place within a cell
-    const int ly0 = ((pyl + 7) >> 3) - 4, lx0 = ((pxl + 7) >> 3) - 4;
+    const int ly0 = cyl - 4, lx0 = cxl - 4;
+    const int nby = ly0 >> lq, nbx = lx0 >> lq;  // the first superblock around it
     const uint32_t* const lobe = s.lobe + (((-pyl & 7) * 8 + (-pxl & 7)) << 6);
     const bool up = f > 0.f;
     float bound = -INFINITY;
-    uint32_t e16[DIRECT ? kOwn : 1];
-    float2 e[DIRECT ? 1 : kOwn], mx[DIRECT ? 1 : kOwn];
+    // the cells around the peak first: behind the candidates' loads they would
+    // wait for those
+    constexpr int kNearU = 2;  // cells at a time
+    int no[kNearU];
+    float2 nu[kNearU];
+    uint32_t nw[kNearU];
+    const int nsy = nby + nq / nb, nsx = nbx + nq % nb;
+    const bool near_in = !DIRECT && nq < nb * nb && nsy >= 0 && nsx >= 0 && nsy < g.nsy &&
+                         nsx < g.nsx;
+    auto near_load = [&](int c) {
+#pragma unroll
+      for (int j = 0; j < kNearU; ++j) {
+        const int k = c + j * nL;
+        const int cy = (nsy << lq) + (k >> lq), cx = (nsx << lq) + (k & (Q - 1));
+        no[j] = near_in && k < (1 << (2 * lq)) && cy < g.ncy && cx < g.ncx ? cy * g.pitch + cx : -1;
+        if (no[j] < 0) continue;
+        nu[j] = ld_cell(&g.u[no[j]]);
+        nw[j] = (unsigned)(cy - ly0) < 8u && (unsigned)(cx - lx0) < 8u
+                    ? lobe[(cy - ly0) * 8 + cx - lx0]
+                    : ld_range(d.sel.h8 + ((cy + d.sel.oy8) * d.sel.w8 + cx + d.sel.ox8 + h0));
+      }
+    };
+    if (near_warp) near_load(nc0);
+    uint32_t e16[kOwn];
+    float2 mx[DIRECT ? 1 : kOwn];
 #pragma unroll
     for (int i = 0; i < kOwn; ++i) {
       if (i * kThreads >= ns) break;
       if (DIRECT) {
-        e16[i] = hbd[hb0 + hbi[i]];
+        e16[i] = h8s[h0 + hbi[i]];
         if (e16[i] == kLobeMark) {
           const int c = tid + i * kThreads, cy = c / g.nsx;
           e16[i] = lobe[(cy - ly0) * 8 + c - cy * g.nsx - lx0];
         }
       } else {
-        const uint2 w = hbt[hb0 + hbi[i]];
-        e[i] = make_float2(__uint_as_float(w.x), __uint_as_float(w.y));
+        e16[i] = ld_range(d.sel.hb + h0 + hbi[i]);
         mx[i] = s.M[tid + i * kThreads];
       }
     }
@@ -849,56 +865,48 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
     for (int i = 0; i < kOwn; ++i) {
       const int b = tid + i * kThreads;
       if (i * kThreads >= ns) break;
+      const uint32_t w = up ? e16[i] : __byte_perm(e16[i], 0u, 0x1032);
       if (DIRECT) {
-        const uint32_t w = up ? e16[i] : __byte_perm(e16[i], 0u, 0x1032);
         acc[i].x = __fmaf_ru(m, __uint_as_float(w << 16), acc[i].x);
         acc[i].y = __fmaf_ru(m, __uint_as_float(w & 0xffff0000u), acc[i].y);
         bound = fmaxf(bound, fmaxf(acc[i].x, acc[i].y));
-      } else if (b < ns && e[i].x + e[i].y >= 0.f) {
-        acc[i].x = __fmaf_ru(m, up ? e[i].x : e[i].y, acc[i].x);
-        acc[i].y = __fmaf_ru(m, up ? e[i].y : e[i].x, acc[i].y);
+      } else if (b < ns &&
+                 !((unsigned)(sby[i] - nby) < (unsigned)nb && (unsigned)(sbx[i] - nbx) < (unsigned)nb)) {
+        acc[i].x = __fmaf_ru(m, __uint_as_float(w << 16), acc[i].x);
+        acc[i].y = __fmaf_ru(m, __uint_as_float(w & 0xffff0000u), acc[i].y);
         s.acc[b] = acc[i];
         const float2 a = add_ru(acc[i], mx[i]);
         bound = fmaxf(bound, fmaxf(a.x, a.y));
       }
     }
-    // ---- the cells of those 4 x 4 superblocks one by one ----
-    if (!DIRECT) {
-      const int cy0 = (cyl - 2) << lq, cx0 = (cxl - 2) << lq;  // their first cell
+    // ---- the cells of the superblocks around the peak one by one ----
+    if (near_warp) {
+      float2 mm = make_float2(-INFINITY, -INFINITY);
 #pragma unroll 1
-      for (int q = nq0; q < 16; q += kThreads >> nlw) {
-        const int by = cyl - 2 + (q >> 2), bx = cxl - 2 + (q & 3), b = by * g.nsx + bx;
-        const bool in = by >= 0 && bx >= 0 && by < g.nsy && bx < g.nsx;
-        float2 mm = make_float2(-INFINITY, -INFINITY);
-#pragma unroll 1
-        for (int c = nc0; c < (1 << (2 * lq)); c += nL) {
-          const int cy = cy0 + ((q >> 2) << lq) + (c >> lq), cx = cx0 + ((q & 3) << lq) + (c & (Q - 1));
-          if (!in || cy >= g.ncy || cx >= g.ncx) continue;
-          const int o = cy * g.pitch + cx;
-          float2 e;
-          if ((unsigned)(cy - ly0) < 8u && (unsigned)(cx - lx0) < 8u) {
-            const uint32_t w = lobe[(cy - ly0) * 8 + cx - lx0];
-            e = make_float2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
-          } else {
-            e = __ldg(d.sel.h8 + ((cy - ly0 - 4 + d.sel.oy8) * d.sel.w8 + cx - lx0 - 4 + d.sel.ox8));
-          }
-          float2 u = g.u[o];
-          const float ex = up ? e.x : e.y, ey = up ? e.y : e.x;
-          u.x = __fmaf_ru(m, ex, u.x);
-          u.y = __fmaf_ru(m, ey, u.y);
-          g.u[o] = u;
-          mm = max2(mm, u);
+      for (int c = nc0;;) {
+#pragma unroll
+        for (int j = 0; j < kNearU; ++j) {
+          if (no[j] < 0) continue;
+          if (!up) nw[j] = __byte_perm(nw[j], 0u, 0x1032);
+          nu[j].x = __fmaf_ru(m, __uint_as_float(nw[j] << 16), nu[j].x);
+          nu[j].y = __fmaf_ru(m, __uint_as_float(nw[j] & 0xffff0000u), nu[j].y);
+          g.u[no[j]] = nu[j];
+          mm = max2(mm, nu[j]);
         }
-        if (in) {
-          const float2 a = add_ru(mm, s.acc[b]);
-          bound = fmaxf(bound, fmaxf(a.x, a.y));
-        }
-#pragma unroll 1
-        for (int o = nL >> 1; o > 0; o >>= 1)
-          mm = max2(mm, make_float2(__shfl_xor_sync(0xffffffffu, mm.x, o),
-                                    __shfl_xor_sync(0xffffffffu, mm.y, o)));
-        if (in && nc0 == 0) s.M[b] = mm;
+        c += nL * kNearU;
+        if (c >= 1 << (2 * lq)) break;
+        near_load(c);
       }
+      const int b = nsy * g.nsx + nsx;
+      if (near_in) {
+        const float2 a = add_ru(mm, s.acc[b]);
+        bound = fmaxf(bound, fmaxf(a.x, a.y));
+      }
+#pragma unroll 1
+      for (int o = nL >> 1; o > 0; o >>= 1)
+        mm = max2(mm, make_float2(__shfl_xor_sync(0xffffffffu, mm.x, o),
+                                  __shfl_xor_sync(0xffffffffu, mm.y, o)));
+      if (near_in && nc0 == 0) s.M[b] = mm;
     }
     bound = fmaxf(__fadd_ru(bound, E), 0.f);
 #pragma unroll
@@ -974,8 +982,32 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
     }
     if (fail) break;
   }
-  if (mp) __stcg(mp, __fadd_rn(mval, mflux));
   if (tid == 0) d.sel.ctl[t].near = near;
+  __syncthreads();
+  // the records, here and not an iteration at a time (the thread that kept them
+  // came to every barrier some 500 cycles after the others): the list, and the
+  // model, whose pixels' sums are taken in list order by the thread of the
+  // pixel's first component
+  if (tid < n) {
+    const int4 c = s.comp[tid];
+    clean_component cc;
+    cc.y = g.rc.y0 + c.x;
+    cc.x = g.rc.x0 + c.y;
+    cc.flux = __int_as_float(c.z);
+    cc.tile = t;
+    d.rcomps[(int64_t)t * d.cap_round + k0 + tid] = cc;
+    float* q = d.model + (int64_t)cc.y * d.nx + cc.x;
+    float v = __ldcg(q);
+    bool first = true;
+#pragma unroll 4
+    for (int j = 0; j < n; ++j) {
+      const int4 o = s.comp[j];
+      if (o.x != c.x || o.y != c.y) continue;
+      first &= j >= tid;
+      v = __fadd_rn(v, __int_as_float(o.z));
+    }
+    if (first) __stcg(q, v);
+  }
   __syncthreads();
   return n;
 }
@@ -1191,36 +1223,51 @@ __global__ void psf_lobe_kernel(PlanDev d, uint32_t* __restrict__ out) {
   out[e] = pack_rises(m);
 }
 
-// Ranges over 2 x 2 aligned windows of n8 boxes a side: entry (i, j) covers the
-// boxes from n8 (i - o) to n8 (i - o) + 2 n8 - 1 of each axis (what an n8-box
-// wide block can meet wherever the peak lies), as far as the box table goes.
-// Stored as (-minimum, maximum): the largest rises of R and of -R when the PSF
-// is subtracted once; mark 2: as two bf16, kLobeMark for the 8 x 8 around
-// offset 0.  mark 1: (-1, -1) for the windows around offset 0 (i - o in
-// -2 .. 1).
-__global__ void psf_window_kernel(const float2* __restrict__ g8, int rows8, int cols8, int oy8,
-                                  int ox8, float2* __restrict__ out, int rows, int cols, int oy,
-                                  int ox, int n8, int mark) {
+// Ranges over windows of 2 x 2 boxes: entry (i, j) is what a cell i - oy8 rows
+// and j - ox8 columns of cells from the peak's can meet, wherever in its cell
+// the peak lies.  Stored as the largest rises of R and of -R when the PSF is
+// subtracted once; kLobeMark for the 8 x 8 around offset 0.
+__global__ void psf_window_kernel(const float2* __restrict__ g8, int cols8, int oy8, int ox8,
+                                  uint32_t* __restrict__ out, int rows, int cols) {
   const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (q >= (int64_t)rows * cols) return;
   const int i = (int)(q / cols), j = (int)(q - (int64_t)i * cols);
-  const int y0 = n8 * (i - oy) + oy8, x0 = n8 * (j - ox) + ox8;
-  float2 m = make_float2(0.f, 0.f);
-  bool any = false;
-  for (int y = max(y0, 0); y < min(y0 + 2 * n8, rows8); ++y)
-    for (int x = max(x0, 0); x < min(x0 + 2 * n8, cols8); ++x) {
-      const float2 v = __ldg(&g8[(int64_t)y * cols8 + x]);
-      m.x = any ? fminf(m.x, v.x) : v.x;
-      m.y = any ? fmaxf(m.y, v.y) : v.y;
-      any = true;
-    }
-  if (mark == 2) {
-    const bool lobe = i - oy >= -4 && i - oy < 4 && j - ox >= -4 && j - ox < 4;
-    reinterpret_cast<uint32_t*>(out)[q] = lobe ? kLobeMark : pack_rises(m);
-    return;
+  const float2* b = g8 + (int64_t)i * cols8 + j;  // (the boxes have a row and a column more)
+  const float2 v0 = __ldg(b), v1 = __ldg(b + 1), v2 = __ldg(b + cols8), v3 = __ldg(b + cols8 + 1);
+  const float2 m = make_float2(fminf(fminf(v0.x, v1.x), fminf(v2.x, v3.x)),
+                               fmaxf(fmaxf(v0.y, v1.y), fmaxf(v2.y, v3.y)));
+  const bool lobe = i - oy8 >= -4 && i - oy8 < 4 && j - ox8 >= -4 && j - ox8 < 4;
+  out[q] = lobe ? kLobeMark : pack_rises(m);
+}
+
+// The same for superblocks of n x n cells: windows of n + 1 boxes a side as far
+// as the boxes go, along the rows first (into tmp, `cols` wide), then down the
+// columns.
+__global__ void psf_window_x_kernel(const float2* __restrict__ g8, int rows8, int cols8,
+                                    float2* __restrict__ tmp, int cols, int n) {
+  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= (int64_t)rows8 * cols) return;
+  const int i = (int)(q / cols), j = (int)(q - (int64_t)i * cols);
+  float2 m = make_float2(INFINITY, -INFINITY);
+#pragma unroll 4
+  for (int x = j; x <= min(j + n, cols8 - 1); ++x) {
+    const float2 v = __ldg(&g8[(int64_t)i * cols8 + x]);
+    m = make_float2(fminf(m.x, v.x), fmaxf(m.y, v.y));
   }
-  const bool near = mark && i - oy >= -2 && i - oy <= 1 && j - ox >= -2 && j - ox <= 1;
-  out[q] = near ? make_float2(-1.f, -1.f) : make_float2(-m.x, m.y);
+  tmp[q] = m;
+}
+__global__ void psf_window_y_kernel(const float2* __restrict__ tmp, int rows8, int cols,
+                                    uint32_t* __restrict__ out, int rows, int n) {
+  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= (int64_t)rows * cols) return;
+  const int i = (int)(q / cols), j = (int)(q - (int64_t)i * cols);
+  float2 m = make_float2(INFINITY, -INFINITY);
+#pragma unroll 4
+  for (int y = i; y <= min(i + n, rows8 - 1); ++y) {
+    const float2 v = __ldg(&tmp[(int64_t)y * cols + j]);
+    m = make_float2(fminf(m.x, v.x), fmaxf(m.y, v.y));
+  }
+  out[q] = pack_rises(m);
 }
 
 }  // namespace
@@ -1244,35 +1291,35 @@ bool select_geometry(SelDev* g, int ny, int nx, int ty, int tx, SelSizes* z) {
   g->oy8 = ncy;
   g->ox8 = ncx;
   g->w8 = 2 * ncx + 1;
-  const int nsy = (ncy + (1 << lq) - 1) >> lq, nsx = (ncx + (1 << lq) - 1) >> lq;
-  g->oyb = nsy;
-  g->oxb = nsx;
-  g->wb = 2 * nsx + 1;
-  const size_t entries = (size_t)(2 * nsy + 1) * (size_t)(2 * nsx + 1);
-  z->smem = (int)(sizeof(SelShared) +
-                  (lq > 0 ? sizeof(float2) * entries : (sizeof(uint32_t) * (entries + 1)) & ~7ull));
+  const size_t entries = (size_t)(2 * ncy + 1) * (size_t)(2 * ncx + 1);
+  const size_t boxes = (size_t)(2 * ncy + 2) * (size_t)(2 * ncx + 2);
+  const size_t table = (sizeof(uint32_t) * (entries + 1)) & ~(size_t)7;  // read 8 bytes at a time
+  z->smem = (int)(sizeof(SelShared) + (lq == 0 ? table : 0));
   z->cells = sizeof(float2) * (size_t)g->cell_stride * (size_t)(ty * tx);
-  z->boxes = sizeof(float2) * (size_t)(2 * ncy + 2) * (size_t)(2 * ncx + 2);
-  z->h8 = sizeof(float2) * (size_t)(2 * ncy + 1) * (size_t)(2 * ncx + 1);
-  z->hb = sizeof(float2) * entries;
+  z->boxes = sizeof(float2) * boxes * (lq > 0 ? 2 : 1);  // and the windows' rows
+  z->h8 = table;
+  z->hb = lq > 0 ? table : 0;
   z->lobe = sizeof(uint32_t) * 64 * 64;
   z->ctl = sizeof(SelCtl) * (size_t)(ty * tx);
   return true;
 }
 
-cudaError_t select_build_psf(const PlanDev& d, float2* boxes, float2* h8, float2* hb,
+cudaError_t select_build_psf(const PlanDev& d, float2* boxes, uint32_t* h8, uint32_t* hb,
                              uint32_t* lobe, cudaStream_t s) {
   const SelDev& g = d.sel;
-  const int rows8 = 2 * g.oy8 + 2, cols8 = 2 * g.ox8 + 2;
+  const int rows8 = 2 * g.oy8 + 2, cols8 = 2 * g.ox8 + 2, rows = rows8 - 1, cols = cols8 - 1;
   const int64_t warps = (int64_t)rows8 * ((cols8 + 3) / 4);
+  auto blocks = [](int64_t n) { return (unsigned)((n + 127) / 128); };
   psf_box_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(d, boxes, rows8, cols8);
-  auto windows = [&](float2* out, int oy, int ox, int n8, int mark) {
-    const int64_t n = (int64_t)(2 * oy + 1) * (2 * ox + 1);
-    psf_window_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(
-        boxes, rows8, cols8, g.oy8, g.ox8, out, 2 * oy + 1, 2 * ox + 1, oy, ox, n8, mark);
-  };
-  windows(h8, g.oy8, g.ox8, 1, 0);
-  windows(hb, g.oyb, g.oxb, 1 << g.lq, g.lq > 0 ? 1 : 2);
+  psf_window_kernel<<<blocks((int64_t)rows * cols), 128, 0, s>>>(boxes, cols8, g.oy8, g.ox8, h8,
+                                                                 rows, cols);
+  if (g.lq > 0) {
+    float2* tmp = boxes + (int64_t)rows8 * cols8;
+    psf_window_x_kernel<<<blocks((int64_t)rows8 * cols), 128, 0, s>>>(boxes, rows8, cols8, tmp,
+                                                                      cols, 1 << g.lq);
+    psf_window_y_kernel<<<blocks((int64_t)rows * cols), 128, 0, s>>>(tmp, rows8, cols, hb, rows,
+                                                                     1 << g.lq);
+  }
   psf_lobe_kernel<<<32, 128, 0, s>>>(d, lobe);
   return cudaGetLastError();
 }
