@@ -171,6 +171,14 @@ def _stream_ptr(stream):
     return ctypes.c_void_p(stream.cuda_stream)
 
 
+def _components(comps, n):
+    """The first n rows of a CUDA int32 array of components as a structured
+    array (the rows are the records, so they are copied once)."""
+    if n == 0:
+        return np.empty(0, dtype=COMPONENT_DTYPE)
+    return comps[:n].cpu().numpy().view(COMPONENT_DTYPE).reshape(n)
+
+
 def _dptr(t, shape=None, what="tensor"):
     import torch
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
@@ -295,11 +303,7 @@ class Plan:
         cnt = ctypes.c_int64(0)
         _check(lib().clean_get(self._h, _dptr(res), _dptr(mod), ctypes.c_void_p(comps.data_ptr()),
                                n, ctypes.byref(cnt), _stream_ptr(stream)), "clean_get")
-        host = comps[:n].cpu().numpy()
-        arr = np.empty(n, dtype=COMPONENT_DTYPE)
-        arr["y"], arr["x"], arr["tile"] = host[:, 0], host[:, 1], host[:, 3]
-        arr["flux"] = host[:, 2].view(np.float32)
-        return res, mod, arr
+        return res, mod, _components(comps, n)
 
     def round_offsets(self, stream=None) -> np.ndarray:
         n = ctypes.c_int64(0)
@@ -416,20 +420,16 @@ class Batch:
     def get(self, i, stream=None):
         import torch
         ny, nx = self.shapes[i]
-        n = ctypes.c_int64(0)
-        _check(lib().clean_batch_get(self._h, int(i), None, None, None, 0, ctypes.byref(n),
-                                     _stream_ptr(stream)), "clean_batch_get")
+        n, sp = ctypes.c_int64(0), _stream_ptr(stream)
+        _check(lib().clean_batch_get(self._h, int(i), None, None, None, 0, ctypes.byref(n), sp),
+               "clean_batch_get")
         res = torch.empty((ny, nx), dtype=torch.float32, device="cuda")
         mod = torch.empty_like(res)
         comps = torch.empty((max(n.value, 1), 4), dtype=torch.int32, device="cuda")
         _check(lib().clean_batch_get(self._h, int(i), _dptr(res), _dptr(mod),
                                      ctypes.c_void_p(comps.data_ptr()), n.value, ctypes.byref(n),
-                                     _stream_ptr(stream)), "clean_batch_get")
-        host = comps[:n.value].cpu().numpy()
-        arr = np.empty(n.value, dtype=COMPONENT_DTYPE)
-        arr["y"], arr["x"], arr["tile"] = host[:, 0], host[:, 1], host[:, 3]
-        arr["flux"] = host[:, 2].view(np.float32)
-        return res, mod, arr
+                                     sp), "clean_batch_get")
+        return res, mod, _components(comps, n.value)
 
     def graphs(self, enable=None) -> int:
         """Turns CUDA-graph round replay on or off (None: leave as is);

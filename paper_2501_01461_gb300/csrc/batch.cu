@@ -67,6 +67,7 @@ struct clean_engine_s {
   std::vector<int> free_slots;
   DevState* d_states = nullptr;         // [cap] control blocks
   DevState* h_states = nullptr;         // pinned mirror
+  bool states_read = false;             // it is as the device's: nothing launched since
   PlanDev* d_plans = nullptr;           // [cap] device copies, indexed by work position
   BatchItem* d_items = nullptr;
   int items_cap = 0;
@@ -144,6 +145,7 @@ int engine_create(clean_engine_s** out, int cap) {
 // Starts (or restarts) a job's run from a dirty image: control block and
 // peaks cleared, set-up kernel on `s`; the job's rounds count from now.
 int engine_start(clean_engine_s* e, Job& j, const float* d_dirty, cudaStream_t s) {
+  e->states_read = false;
   j.dev.round0 = e->round;
   j.finished = false;
   cudaError_t err = cudaMemsetAsync(j.dev.st, 0, sizeof(DevState), s);
@@ -343,6 +345,7 @@ int engine_read(clean_engine_s* e, cudaStream_t s) {
                                     cudaMemcpyDeviceToHost, s);
   if (err == cudaSuccess) err = cudaStreamSynchronize(s);
   if (err != cudaSuccess) return eng_fail(e, CLEAN_ERR_CUDA);
+  e->states_read = true;
   bool timeout = false;
   for (const Job& j : e->jobs) {
     const DevState& st = e->h_states[j.slot];
@@ -441,6 +444,7 @@ bool capture_pair(clean_engine_s* e, int par) {
 
 int engine_rounds(clean_engine_s* e, int64_t rounds, cudaStream_t s) {
   int rc;
+  e->states_read = false;
   if (e->dirty && (rc = engine_rebuild(e, s)) != CLEAN_OK) return rc;
   if (e->n_work == 0) return CLEAN_OK;
   while (rounds >= 2 && e->use_graphs && !e->graphs_refused) {
@@ -482,12 +486,14 @@ int engine_get(clean_engine_s* e, const Job& j, float* d_residual, float* d_mode
     err = cudaMemcpyAsync(d_model, j.dev.model, img, cudaMemcpyDeviceToDevice, s);
   if (err != cudaSuccess) return eng_fail(e, CLEAN_ERR_CUDA);
   if (d_comps || n_comps) {
-    DevState st;
-    err = cudaMemcpyAsync(&st, j.dev.st, sizeof(DevState), cudaMemcpyDeviceToHost, s);
+    // (the length is known when nothing was launched since the last read)
+    int64_t total = e->h_states[j.slot].total;
+    if (!e->states_read)
+      err = cudaMemcpyAsync(&total, &j.dev.st->total, sizeof(total), cudaMemcpyDeviceToHost, s);
     if (err == cudaSuccess) err = cudaStreamSynchronize(s);
     if (err != cudaSuccess) return eng_fail(e, CLEAN_ERR_CUDA);
-    if (n_comps) *n_comps = st.total;
-    const int64_t m = std::min(st.total, comps_cap);
+    if (n_comps) *n_comps = total;
+    const int64_t m = std::min(total, comps_cap);
     if (d_comps && m > 0) {
       err = cudaMemcpyAsync(d_comps, j.dev.list, sizeof(clean_component) * (size_t)m,
                             cudaMemcpyDeviceToDevice, s);

@@ -64,9 +64,9 @@ struct clean_plan_s {
   bool pending = false;
   int parity = 0;
   int64_t rounds_launched = 0;
-  DevState* h_st = nullptr;
+  DevState h_st{};            // mirror of the control block (read_state)
   float* beam_buf = nullptr;
-  std::vector<void*> allocs;
+  void* arena = nullptr;      // the allocation that holds every array of the plan
   // launch accounting and optional per-launch CUDA-event timing
   int64_t kernel_launches = 0;
   bool timing = false;
@@ -205,14 +205,15 @@ void timed_collect(clean_plan_s* pl) {
   pl->ev_kind.clear();
 }
 
-// Reads the device control block into the pinned mirror (synchronises).
+// Reads the device control block into its mirror (synchronises).  96 bytes: a
+// copy to ordinary memory takes 9 us, to pinned memory 8.
 int read_state(clean_plan_s* pl, cudaStream_t s) {
-  cudaError_t e = cudaMemcpyAsync(pl->h_st, pl->d.st, sizeof(DevState),
+  cudaError_t e = cudaMemcpyAsync(&pl->h_st, pl->d.st, sizeof(DevState),
                                   cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return cuda_fail(pl, e);
   timed_collect(pl);
-  if (pl->h_st->status & ST_TIMEOUT) return poison(pl, CLEAN_ERR_TIMEOUT);
+  if (pl->h_st.status & ST_TIMEOUT) return poison(pl, CLEAN_ERR_TIMEOUT);
   return CLEAN_OK;
 }
 
@@ -246,7 +247,7 @@ int check_psf(clean_plan_s* pl, cudaStream_t s) {
   if (e != cudaSuccess) return cuda_fail(pl, e);
   int rc = read_state(pl, s);
   if (rc != CLEAN_OK) return rc;
-  const int bits = pl->h_st->status;
+  const int bits = pl->h_st.status;
   pl->psf_set = true;
   pl->psf_status = (bits & ST_NONFINITE_PSF)   ? CLEAN_ERR_NONFINITE
                    : (bits & ST_PSF_OFFCENTRE) ? CLEAN_ERR_INVALID_ARG
@@ -507,15 +508,15 @@ int run_rounds(clean_plan_s* pl, int32_t max_rounds, cudaStream_t s) {
   int rc;
   if (pl->pending && (rc = launch_round_feedback(pl, s)) != CLEAN_OK) return rc;
   if ((rc = read_state(pl, s)) != CLEAN_OK) return rc;
-  if (pl->h_st->status & ST_NONFINITE_DIRTY) {
+  if (pl->h_st.status & ST_NONFINITE_DIRTY) {
     pl->started = false;
     return CLEAN_ERR_NONFINITE;
   }
   int64_t done = 0;
   while (max_rounds < 0 || done < max_rounds) {
-    if (!pl->h_st->active) break;
+    if (!pl->h_st.active) break;
     int64_t chunk = 1;
-    if (pl->d.K > 0) chunk = (pl->h_st->max_budget + pl->d.K - 1) / pl->d.K;
+    if (pl->d.K > 0) chunk = (pl->h_st.max_budget + pl->d.K - 1) / pl->d.K;
     chunk = std::max<int64_t>(chunk, 1);
     if (max_rounds >= 0) chunk = std::min<int64_t>(chunk, max_rounds - done);
     NvtxRange range("clean_rounds");
@@ -624,11 +625,10 @@ void clean_destroy(clean_plan_t pl) {
     cudaDeviceSynchronize();
     drop_graphs(pl);
     if (pl->cap_stream) cudaStreamDestroy(pl->cap_stream);
-    for (void* a : pl->allocs) cudaFree(a);
+    if (pl->arena) cudaFree(pl->arena);
     for (cudaEvent_t e : pl->ev_pool) cudaEventDestroy(e);
     for (cudaEvent_t e : pl->host_ev)
       if (e) cudaEventDestroy(e);
-    if (pl->h_st) cudaFreeHost(pl->h_st);
     cudaGetLastError();
   }
   delete pl;
@@ -836,22 +836,22 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
     delete pl;
     return CLEAN_ERR_OOM;
   }
-  for (auto& r : req) {
-    void* ptr = nullptr;
-    if (cudaMalloc(&ptr, r.bytes) != cudaSuccess) {
-      cudaGetLastError();
-      clean_destroy(pl);
-      return CLEAN_ERR_OOM;
-    }
-    pl->allocs.push_back(ptr);
-    *r.dst = ptr;
-  }
-  if (cudaMallocHost((void**)&pl->h_st, sizeof(DevState)) != cudaSuccess) {
+  // one allocation, each array at a multiple of 256 bytes: a server makes a plan
+  // per job, and twenty allocations and a page of pinned memory cost it 0.3 ms
+  // (0.17 + 0.14) and their release 0.35; one costs 0.08 and 0.05
+  size_t arena = 0;
+  for (auto& r : req) arena += (r.bytes + 255) & ~(size_t)255;
+  if (cudaMalloc(&pl->arena, arena) != cudaSuccess) {
+    pl->arena = nullptr;
     cudaGetLastError();
     clean_destroy(pl);
     return CLEAN_ERR_OOM;
   }
-  std::memset(pl->h_st, 0, sizeof(DevState));
+  char* at = static_cast<char*>(pl->arena);
+  for (auto& r : req) {
+    *r.dst = at;
+    at += (r.bytes + 255) & ~(size_t)255;
+  }
 
   PlanDev& d = pl->d;
   d.P = d_psf ? d_psf : pl->psf_own;
@@ -989,7 +989,7 @@ int clean_get(clean_plan_t pl, float* d_residual_out, float* d_model_out,
   if (d_comps_out || n_comps) {
     int rc = read_state(pl, s);
     if (rc != CLEAN_OK) return rc;
-    const int64_t n = pl->h_st->total;
+    const int64_t n = pl->h_st.total;
     if (n_comps) *n_comps = n;
     if (d_comps_out) {
       const int64_t m = std::min(n, comps_cap);
@@ -1012,7 +1012,7 @@ int clean_get_rounds(clean_plan_t pl, int64_t* h_offsets, int64_t cap, int64_t* 
   cudaStream_t s = as_stream(stream);
   int rc = read_state(pl, s);
   if (rc != CLEAN_OK) return rc;
-  const int64_t n = pl->h_st->n_rounds;
+  const int64_t n = pl->h_st.n_rounds;
   if (n_rounds) *n_rounds = n;
   if (h_offsets && cap > 0 && n > 0) {
     const int64_t m = std::min(n, cap);
@@ -1076,7 +1076,7 @@ int clean_checkpoint(clean_plan_t pl, void* h_buf, int64_t capacity, int64_t* by
   cudaStream_t s = as_stream(stream);
   int rc = read_state(pl, s);
   if (rc != CLEAN_OK) return rc;
-  const DevState st = *pl->h_st;
+  const DevState st = pl->h_st;
   const int64_t npix = (int64_t)pl->d.ny * pl->d.nx;
   const int64_t need = ckpt_bytes(npix, pl->d.T, st.total, st.n_rounds);
   *bytes = need;
@@ -1178,7 +1178,7 @@ int clean_deconvolve_host(clean_plan_t pl, const float* h_dirty, const float* h_
   if (e == cudaSuccess && h_model)
     e = cudaMemcpyAsync(h_model, pl->d.model, img, cudaMemcpyDeviceToHost, s);
   if (e != cudaSuccess) return cuda_fail(pl, e);
-  const int64_t n = pl->h_st->total;  // read by run_rounds' last status read
+  const int64_t n = pl->h_st.total;  // read by run_rounds' last status read
   if (n_comps) *n_comps = n;
   if (h_comps && comps_cap > 0 && n > 0) {
     e = cudaMemcpyAsync(h_comps, pl->d.list,
@@ -1221,8 +1221,8 @@ int clean_stats(clean_plan_t pl, clean_stats_t* out, void* stream) {
   DeviceGuard g(pl->device);
   int rc = read_state(pl, as_stream(stream));
   if (rc != CLEAN_OK) return rc;
-  out->n_components = pl->h_st->total;
-  out->rounds = pl->h_st->n_rounds;
+  out->n_components = pl->h_st.total;
+  out->rounds = pl->h_st.n_rounds;
   out->minor_launches = pl->minor_launches;
   out->feedback_launches = pl->feedback_launches;
   out->minor_ms = pl->minor_ms;

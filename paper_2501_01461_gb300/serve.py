@@ -20,7 +20,7 @@ from dataclasses import dataclass, field
 
 import numpy as np
 
-from . import (COMPONENT_DTYPE, FB_FFT, FB_GATHER, CleanError, _check, _dptr, _stream_ptr,
+from . import (FB_FFT, FB_GATHER, CleanError, _check, _components, _dptr, _stream_ptr,
                lib, make_params)
 
 
@@ -150,20 +150,16 @@ class Server:
 
     def get(self, jid: int, shape):
         import torch
-        n = ctypes.c_int64(0)
-        _check(lib().clean_server_get(self._h, jid, None, None, None, 0, ctypes.byref(n),
-                                      _stream_ptr(self._stream)), "clean_server_get")
+        n, sp = ctypes.c_int64(0), _stream_ptr(self._stream)
+        _check(lib().clean_server_get(self._h, jid, None, None, None, 0, ctypes.byref(n), sp),
+               "clean_server_get")
         res = torch.empty(shape, dtype=torch.float32, device="cuda")
         mod = torch.empty_like(res)
         comps = torch.empty((max(n.value, 1), 4), dtype=torch.int32, device="cuda")
         _check(lib().clean_server_get(self._h, jid, _dptr(res), _dptr(mod),
                                       ctypes.c_void_p(comps.data_ptr()), n.value, ctypes.byref(n),
-                                      _stream_ptr(self._stream)), "clean_server_get")
-        host = comps[:n.value].cpu().numpy()
-        arr = np.empty(n.value, dtype=COMPONENT_DTYPE)
-        arr["y"], arr["x"], arr["tile"] = host[:, 0], host[:, 1], host[:, 3]
-        arr["flux"] = host[:, 2].view(np.float32)
-        return res, mod, arr
+                                      sp), "clean_server_get")
+        return res, mod, _components(comps, n.value)
 
     def remove(self, jid: int):
         _check(lib().clean_server_remove(self._h, jid), "clean_server_remove")
