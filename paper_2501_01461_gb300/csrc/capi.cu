@@ -515,8 +515,18 @@ int run_rounds(clean_plan_s* pl, int32_t max_rounds, cudaStream_t s) {
   int64_t done = 0;
   while (max_rounds < 0 || done < max_rounds) {
     if (!pl->h_st.active) break;
-    int64_t chunk = 1;
-    if (pl->d.K > 0) chunk = (pl->h_st.max_budget + pl->d.K - 1) / pl->d.K;
+    // rounds until the next status read: all that the budget can need, unless a
+    // threshold or the flux trigger may end the run (or a round) before.  An
+    // empty round costs about 7 us, a read 15 with the gap it leaves: eight at
+    // first, then half of those done so far (1024^2 to five sigma, some 20 rounds of
+    // 50 possible: 3.88 ms with one read, now 3.71); four for rounds that the
+    // trigger ends (301 x 277, eight rounds: 1.49 ms with a read each, now 1.38)
+    const int64_t left = pl->h_st.max_budget;
+    int64_t chunk = pl->d.K > 0 ? (left + pl->d.K - 1) / pl->d.K : 1;
+    if (pl->d.trigger > 0.f)
+      chunk = std::min(std::max<int64_t>(4, done / 2), left);
+    else if (pl->d.thr > 0.f)
+      chunk = std::min(chunk, std::max<int64_t>(8, done / 2));
     chunk = std::max<int64_t>(chunk, 1);
     if (max_rounds >= 0) chunk = std::min<int64_t>(chunk, max_rounds - done);
     NvtxRange range("clean_rounds");
