@@ -42,11 +42,13 @@
 // 4 x 4 cells), not of 4 x 4.  It does not fit shared memory and need not: its
 // L2 round trip runs beside the candidates'.
 //
-// What bounds it: an iteration is a chain of about 1400 cycles (0.7 us: decode,
+// What bounds it: an iteration is a chain of about 1500 cycles (0.75 us: decode,
 // one L2 round trip of the candidates' PSF gather at one L1 tag a candidate,
-// two warp reductions either side of a barrier), whatever the tile's size; the
-// plain loop's were 3.3 us (256^2, cluster of 16) to 12 us (sixteen 1024^2
-// tiles).  Code size matters: straight-line code beyond the 32 KB that stay
+// two warp reductions either side of a barrier), 3400 with superblocks (the
+// gather misses L1 there, and the cells near the peak come after it); the
+// plain loop's were 3.3 us (256^2, cluster of 16) to 12 us (2048^2, and sixteen
+// 1024^2 tiles at once).  On a flat residual the resolved cells' gathers take as
+// long again.  Code size matters: straight-line code beyond the 32 KB that stay
 // near the schedulers ran at a third of the speed, so the rare parts are
 // rolled loops.
 #include <algorithm>
@@ -202,8 +204,14 @@ __device__ __forceinline__ bool psf_at(const PlanDev& d, int sy, int sx, float* 
   return in;
 }
 
-// Two pixels' values less n pending components, in order (32 PSF loads in
-// flight).
+// The same as one index of the array, below 0 outside.
+__device__ __forceinline__ int psf_index(const PlanDev& d, int sy, int sx) {
+  return (unsigned)sy < (unsigned)d.pny && (unsigned)sx < (unsigned)d.pnx ? sy * d.pnx + sx : -1;
+}
+
+// Two pixels' values less n pending components, in order (up to 32 PSF loads
+// in flight; one component at a time, as the clipped PSF had it first, a
+// 256 x 256 image with a PSF no larger took 34 ms for 8000 iterations).
 __device__ __forceinline__ void less_pending(const PlanDev& d, float (&r)[2],
                                              const uint32_t (&pos)[2], int n) {
   SelShared& s = shared_state();
@@ -234,13 +242,28 @@ __device__ __forceinline__ void less_pending(const PlanDev& d, float (&r)[2],
       }
     }
   } else {
+    // (the array's first value stands in for one off the array)
+    constexpr int U = 8;
 #pragma unroll 1
-    for (int j = 0; j < n; ++j) {
-      const int4 c = s.comp[j];
-      const float f = __int_as_float(c.z);
-      float q;
-      if (psf_at(d, y0 - c.x + d.cy, x0 - c.y + d.cx, &q)) r[0] = __fsub_rn(r[0], __fmul_rn(f, q));
-      if (psf_at(d, y1 - c.x + d.cy, x1 - c.y + d.cx, &q)) r[1] = __fsub_rn(r[1], __fmul_rn(f, q));
+    for (int j0 = 0; j0 < n; j0 += U) {
+      float p[U][2];
+      uint32_t in = 0u;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int4 c = s.comp[j0 + u];
+        const int cy = d.cy - c.x, cx = d.cx - c.y;
+        const int o0 = psf_index(d, y0 + cy, x0 + cx), o1 = psf_index(d, y1 + cy, x1 + cx);
+        in |= (uint32_t)(o0 >= 0 && j0 + u < n) << (2 * u);
+        in |= (uint32_t)(o1 >= 0 && j0 + u < n) << (2 * u + 1);
+        p[u][0] = ptx::ld_nc(d.P + max(o0, 0));
+        p[u][1] = ptx::ld_nc(d.P + max(o1, 0));
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const float f = __int_as_float(s.comp[j0 + u].z);
+        if ((in >> (2 * u)) & 1u) r[0] = __fsub_rn(r[0], __fmul_rn(f, p[u][0]));
+        if ((in >> (2 * u + 1)) & 1u) r[1] = __fsub_rn(r[1], __fmul_rn(f, p[u][1]));
+      }
     }
   }
 }
@@ -312,18 +335,28 @@ __device__ __forceinline__ void tile_pass(const PlanDev& d, const Geo& g, int ra
           }
         }
       } else {
+        constexpr int U = 4;
 #pragma unroll 1
-        for (int j = 0; j < n; ++j) {
-          const int4 c = s.comp[j];
-          const float f = __int_as_float(c.z);
-          float p[kUnitRows];
-          bool ok[kUnitRows];
+        for (int j = 0; j < n; j += U) {
+          float p[U][kUnitRows];
+          uint32_t in = 0u;
 #pragma unroll
-          for (int i = 0; i < kUnitRows; ++i)
-            ok[i] = psf_at(d, ly + i - c.x + d.cy, lx - c.y + d.cx, &p[i]);
+          for (int u = 0; u < U; ++u) {
+            const int4 c = s.comp[j + u];
 #pragma unroll
-          for (int i = 0; i < kUnitRows; ++i)
-            if (ok[i]) r[i] = __fsub_rn(r[i], __fmul_rn(f, p[i]));
+            for (int i = 0; i < kUnitRows; ++i) {
+              const int o = psf_index(d, ly + i - c.x + d.cy, lx - c.y + d.cx);
+              in |= (uint32_t)(o >= 0 && j + u < n) << (u * kUnitRows + i);
+              p[u][i] = ptx::ld_nc(d.P + max(o, 0));
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            const float f = __int_as_float(s.comp[j + u].z);
+#pragma unroll
+            for (int i = 0; i < kUnitRows; ++i)
+              if ((in >> (u * kUnitRows + i)) & 1u) r[i] = __fsub_rn(r[i], __fmul_rn(f, p[u][i]));
+          }
         }
       }
 #pragma unroll
