@@ -222,28 +222,21 @@ def aggregate(dist, ms: float, units: float, device=None):
 
 
 def minor_bytes_per_run(w) -> int:
-    """Algorithmic bytes of all minor iterations of one run: each iteration of
-    tile t reads its M_t residual pixels and the M_t-pixel PSF window and
-    writes M_t residual pixels (12 M_t bytes)."""
-    ty, tx = w.tiles
-    T = ty * tx
-    M = [((i + 1) * w.n // ty - i * w.n // ty) * ((j + 1) * w.n // tx - j * w.n // tx)
-         for i in range(ty) for j in range(tx)]
-    per_tile = [w.niter // T + (1 if t < w.niter % T else 0) for t in range(T)]
-    return int(sum(12 * m * k for m, k in zip(M, per_tile)))
+    """Algorithmic bytes of all minor loops of one run: a round's selection
+    reads the residual once (its cells' bounds) and leaves the subtraction to
+    the feedback; the iterations themselves touch a few KB each."""
+    T = w.tiles[0] * w.tiles[1]
+    per_tile = w.niter // T + (1 if w.niter % T else 0)
+    k = w.feedback_interval if w.feedback_interval > 0 else per_tile
+    return int(-(-per_tile // k) * 4 * w.n * w.n)
 
 
 def feedback_updates_per_run(w) -> int:
     """Pixel-component updates of all feedbacks of one run (threshold 0, every
-    tile spends its budget): each component updates every pixel outside its
-    own tile once."""
-    ty, tx = w.tiles
-    T = ty * tx
-    N2 = w.n * w.n
-    M = [((i + 1) * w.n // ty - i * w.n // ty) * ((j + 1) * w.n // tx - j * w.n // tx)
-         for i in range(ty) for j in range(tx)]
-    per_tile = [w.niter // T + (1 if t < w.niter % T else 0) for t in range(T)]
-    return int(sum((N2 - m) * k for m, k in zip(M, per_tile))) if w.feedback_interval > 0 else 0
+    tile spends its budget): each component updates every pixel once, those of
+    its own tile too (the selection leaves a round of up to 64 components
+    pending)."""
+    return int(w.niter * w.n * w.n) if w.feedback_interval > 0 else 0
 
 
 def measured_peaks():
@@ -346,16 +339,15 @@ def batch_leg(cg, torch, stream, n_images=64):
     for p in plain:
         p.close()
     sides = [j["n"] for j in jobs]
-    # algorithmic bytes of one run: minor loop 12 B per pixel-iteration (of
-    # the iteration's tile), feedback 4 B per pixel-component update + 8 N^2
-    # per round; the iteration budget is spent in full (threshold 0)
+    # algorithmic bytes of one run: feedback 4 B per pixel-component update (the
+    # component's own tile too) + 8 N^2 per round, the minor loops 4 N^2 per
+    # round; the iteration budget is spent in full (threshold 0)
     px_iter = bytes_ = 0.0
     for j in jobs:
         n, (ty, tx), nit, K = j["n"], j["tiles"], j["niter"], j["K"]
         T = ty * tx
-        M = n * n / T
-        px_iter += nit * M
-        bytes_ += 12.0 * nit * M + 4.0 * nit * (n * n - M) + 8.0 * n * n * (-(-nit // (K * T)))
+        px_iter += nit * n * n / T
+        bytes_ += 4.0 * nit * n * n + 12.0 * n * n * (-(-nit // (K * T)))
     return {"workload": f"{n_images} images, sides {sorted(set(sides))} (counts "
                         f"{[sides.count(v) for v in sorted(set(sides))]}), PSF 2N, freq scale 1-2, "
                         "2x2 tiles up to 1024 else 4x4, K 50, 2000 iterations each",
@@ -370,8 +362,8 @@ def batch_leg(cg, torch, stream, n_images=64):
             "kernel_launches_per_run": st["kernel_launches"],
             "set_up_launches_per_run": n_images,
             "launches_per_round": (st["kernel_launches"] - n_images) / max(1, st["rounds_launched"]),
-            "note": "per run: one set-up kernel per image, then each round one persistent "
-                    "minor-loop launch over every image's tiles and one feedback launch"}
+            "note": "per run: one set-up kernel per image, then each round one minor-loop "
+                    "launch per kind of tile over every image's tiles and one feedback launch"}
 
 
 def serve_leg(cg, torch, psf_full, n_jobs=60, loads=(0.7,), seed=1004):
@@ -690,8 +682,7 @@ def main():
     alu_peak = st["sm_count"] * 128 * sm_mhz * 1e6 / 1e12
     rec = ncu_traffic()
     traffic = {k: v["bytes_per_launch"] for k, v in rec.items()}
-    minor_name = ("minor_pair_kernel" if st.get("minor_pairs") else "minor_pipe_kernel") \
-        if st["minor_pipe"] else "minor_kernel"
+    minor_name = "select_kernel"
     fb_name = "feedback_tma_kernel" if st["feedback_tma"] else "feedback_kernel"
     l2_src = (f"measured in this run: {l2['form']} ({l2['method']}); MEASURED_PEAKS.json "
               f"holds no L2 figure (its HBM copy peak is {peaks['hbm_gbs']:.0f} GB/s, {peak_src})")
@@ -710,7 +701,8 @@ def main():
         roof = {"kernel": minor_name, "bound": "l2", "achieved": minor_gbs, "peak": l2_gbs,
                 "unit": "GB/s", "frac": minor_gbs / l2_gbs, "traffic": traffic.get(minor_name),
                 "peak_source": l2_src, "bytes_per_launch": minor_b,
-                "note": "12 B per pixel per tile iteration; traffic = DRAM bytes per launch"}
+                "note": "the residual once a round; the launch is bound by the chain of its "
+                        "iterations, not by bytes"}
     kernels = {
         "minor": {"kernel": minor_name,
                   "ms_per_step": st["minor_ms"] / args.steps,
@@ -718,8 +710,11 @@ def main():
                   "bytes_per_launch": minor_b, "algorithmic_GBps": minor_gbs,
                   "frac_of_l2_peak": minor_gbs / l2_gbs,
                   "traffic": traffic.get(minor_name),
-                  "note": "12 B per pixel per tile iteration (read R, read the PSF window, "
-                          "write R) over the measured L2 read peak"},
+                  "us_per_iteration": st["minor_ms"] * 1e3 * w.tiles[0] * w.tiles[1]
+                  / (w.niter * args.steps),
+                  "note": "the residual once a round over the measured L2 read peak; the "
+                          "launch is bound by the chain of its iterations (us_per_iteration: "
+                          "of one tile, all tiles at once)"},
         "feedback": {"kernel": fb_name,
                      "ms_per_step": st["feedback_ms"] / args.steps,
                      "launches_per_step": st["feedback_launches"] / args.steps,

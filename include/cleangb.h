@@ -109,7 +109,7 @@ typedef struct {
   int32_t feedback_interval; /* K >= 0 minor iterations per tile between feedbacks */
   int32_t feedback_mode;     /* CLEAN_FB_GATHER (exact) | CLEAN_FB_FFT | CLEAN_FB_AUTO */
   int32_t mode;              /* CLEAN_TILED | CLEAN_UNTILED_GRID (needs a 1 x 1 grid) */
-  int32_t group_ctas;        /* CTAs per tile in the minor loop; 0 = choose */
+  int32_t group_ctas;        /* CTAs per tile in the minor loop; 0 = choose (by selection) */
   int32_t group_sync;        /* CLEAN_SYNC_*: cluster barrier or bounded grid barrier */
   float feedback_trigger;    /* 0, or in (0, 1): a tile's round also ends once its
                                 |peak| <= feedback_trigger x the largest |peak| among
@@ -288,9 +288,9 @@ CLEAN_API int clean_hogbom_noalloc(const float* d_dirty, const float* d_psf, int
 /* ---- Batches: many images deconvolved together ----------------------
  * A batch holds n independent deconvolutions (each its own dirty image, PSF
  * and clean_params, sizes and tile grids free) and runs all of them round by
- * round in shared launches: one minor-loop launch per residual placement with
- * one CTA per (image, tile), largest tiles first, and one feedback launch over
- * every image's blocks.  The paper treats one image; batching changes only
+ * round in shared launches: one minor-loop launch per kind of tile with one CTA
+ * (or one cluster) per (image, tile), largest tiles first, and one feedback
+ * launch over every image's blocks.  The paper treats one image; batching changes only
  * which CTA serves which tile, so each image's results are bit for bit those
  * of its own clean_plan + clean_run.  Images with FFT feedback (feedback_mode
  * FFT, or AUTO when the plan picks it) share the minor-loop launches and run
@@ -415,10 +415,12 @@ CLEAN_API const char* clean_strerror(int status);
  *                              configuration (not while timing, not for the
  *                              FFT feedback); 0: launch every kernel directly.
  *                              Same results, bit for bit.
- *   CLEAN_DEBUG_MINOR_PATH     minor-loop kernel: 0 automatic (bulk-copy
- *                              pipeline when image and PSF rows are 16-byte
- *                              aligned), 1 plain loads, 2 pipeline when
- *                              possible (same results, bit for bit)
+ *   CLEAN_DEBUG_MINOR_PATH     minor-loop kernel: 0 automatic (selection when
+ *                              group_ctas and group_sync are left to the
+ *                              library and no tile side is above 32767; else
+ *                              the bulk-copy pipeline when image and PSF rows
+ *                              are 16-byte aligned), 1 plain loads, 2 pipeline
+ *                              when possible (same results, bit for bit)
  *   CLEAN_DEBUG_PIPE_CHUNK_PX  pipeline tuning: about this many pixels per
  *                              staged chunk (0: 4096)
  *   CLEAN_DEBUG_PIPE_STAGES    pipeline tuning: at most this many buffers in
