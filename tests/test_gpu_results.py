@@ -60,3 +60,18 @@ def test_arrays_of_odd_sizes_do_not_overlap(ny, nx, tiles, niter):
         assert np.array_equal(a.cpu().numpy(), b.cpu().numpy())
         assert np.array_equal(a.cpu().numpy(), -c.cpu().numpy())
     assert np.array_equal(one[2], two[2]) and np.array_equal(one[2]["y"], neg[2]["y"])
+
+
+def test_deep_run_of_a_small_tile():
+    """A small tile cleaned far into its noise takes the iteration-by-iteration
+    loop; with a threshold that never ends the run, selections."""
+    psf, dirty = _data(72, 56, 5)
+    out = []
+    for thr in (0.0, 1e-30):
+        with cg.Plan(psf, 72, 56, gain=0.1, niter=2500, threshold=thr) as p:
+            p.run(dirty)
+            out.append(p.get())
+    (r0, m0, c0), (r1, m1, c1) = out
+    assert len(c0) == 2500 and np.array_equal(c0, c1)
+    assert np.array_equal(r0.cpu().numpy(), r1.cpu().numpy())
+    assert np.array_equal(m0.cpu().numpy(), m1.cpu().numpy())
