@@ -131,7 +131,7 @@ struct SelShared {
   int hist[kBins], more[kBins];
   uint32_t cells[kResolveMax];  // cells, row << 16 | column
   uint32_t sbs[kMaxSb];         // superblocks, row << 16 | column
-  int n_cells, n_sbs, n_cand, bin;
+  int n_cells, n_sbs, n_cand, n_pix, bin;
   unsigned long long key;     // the pass's peak key (this CTA's part)
   long long k_cmd;            // the group's command: components so far, finished
   int done_cmd, abort;
@@ -529,7 +529,7 @@ __device__ __forceinline__ void list_cells(const Geo& g, uint32_t abs0, int leas
   }
 }
 
-// Counts the listed cells' pixels in bin `least` or above by bin, and in s.n_cand.
+// Counts the listed cells' pixels in bin `least` or above by bin, and in s.n_pix.
 __device__ __forceinline__ void count_pixels(const PlanDev& d, const Geo& g, uint32_t abs0, int nl,
                                              int least) {
   SelShared& s = shared_state();
@@ -544,7 +544,7 @@ __device__ __forceinline__ void count_pixels(const PlanDev& d, const Geo& g, uin
     if (b >= least) atomicAdd(&s.hist[b], 1);
     total += __popc(__ballot_sync(0xffffffffu, b >= least));
   }
-  if (lane == 0 && total) atomicAdd(&s.n_cand, total);
+  if (lane == 0 && total) atomicAdd(&s.n_pix, total);
 }
 
 // The first candidates: the listed cells' pixels in bin `least` or above (they
@@ -713,7 +713,7 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
   for (int i = tid; i < kBins; i += kThreads) s.hist[i] = 0;
   if (!DIRECT)
     for (int b = tid; b < ns; b += kThreads) s.acc[b] = make_float2(0.f, 0.f);
-  if (tid == 0) s.n_cells = s.n_sbs = s.n_cand = 0;
+  if (tid == 0) s.n_cells = s.n_sbs = s.n_cand = s.n_pix = 0;
   for (int i = tid; i < 64 * 64 / 4; i += kThreads)
     reinterpret_cast<uint4*>(s.lobe)[i] = __ldg(reinterpret_cast<const uint4*>(d.sel.lobe) + i);
   if (DIRECT) {
@@ -758,15 +758,15 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
       nl = min(s.n_cells, kMoreCells);
       count_pixels(d, g, abs0, nl, least);
       __syncthreads();
-      if (most == kMoreCells || s.n_cand >= kCandStart / 4 || least == 1) break;
+      // (no thread writes this count before the block's next barrier)
+      if (most == kMoreCells || s.n_pix >= kCandStart / 4 || least == 1) break;
       // too few: back to the cells' counts
       for (int i = tid; i < kBins; i += kThreads) s.hist[i] = s.more[i];
       __syncthreads();
-      if (tid == 0) s.n_cells = s.n_cand = 0;
+      if (tid == 0) s.n_cells = s.n_pix = 0;
       __syncthreads();
     }
     if (warp == 0) pick_bin(kCandStart);
-    if (tid == 0) s.n_cand = 0;
     __syncthreads();
     start_candidates(d, g, abs0, nl, max(s.bin, least));
     __syncthreads();
