@@ -1042,6 +1042,8 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
   // came to every barrier some 500 cycles after the others): the list, and the
   // model, whose pixels' sums are taken in list order by the thread of the
   // pixel's first component
+  float* sum = nullptr;
+  float v = 0.f;
   if (tid < n) {
     const int4 c = s.comp[tid];
     clean_component cc;
@@ -1050,8 +1052,8 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
     cc.flux = __int_as_float(c.z);
     cc.tile = t;
     d.rcomps[(int64_t)t * d.cap_round + k0 + tid] = cc;
-    float* q = d.model + (int64_t)cc.y * d.nx + cc.x;
-    float v = __ldcg(q);
+    sum = d.model + (int64_t)cc.y * d.nx + cc.x;
+    v = __ldcg(sum);
     bool first = true;
 #pragma unroll 4
     for (int j = 0; j < n; ++j) {
@@ -1060,8 +1062,10 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
       first &= j >= tid;
       v = __fadd_rn(v, __int_as_float(o.z));
     }
-    if (first) __stcg(q, v);
+    if (!first) sum = nullptr;
   }
+  __syncthreads();  // every component of a pixel has read it
+  if (sum) __stcg(sum, v);
   __syncthreads();
   return n;
 }

@@ -117,3 +117,13 @@ def test_first_candidates(emulator, tmp_path):
     dirty, psf = _field(64, 64, (128, 128), 64)
     dirty[10, 50], dirty[50, 10] = 3.0, 2.9
     _check(emulator, tmp_path, dirty, psf, 2)
+
+
+@pytest.mark.parametrize("ny,nx,ps,niter,G,threads", [
+    (64, 64, (128, 128), 90, 1, 64),     # cells kept singly; more than one selection
+    (61, 45, (61, 45), 30, 2, 64),       # a group of two, a clipped PSF, ragged cells
+    (40, 56, (81, 113), 70, 3, 128),
+])
+def test_no_races_and_the_oracles_bits(emulator, tmp_path, ny, nx, ps, niter, G, threads):
+    dirty, psf = _field(ny, nx, ps, ny)
+    _check(emulator, tmp_path, dirty, psf, niter, G=G, threads=threads)
