@@ -886,6 +886,7 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
     if (near_warp) near_load(nc0);
     uint32_t e16[kOwn];
     float2 mx[DIRECT ? 1 : kOwn];
+    bool far[DIRECT ? 1 : kOwn];  // not around the peak (those change below)
 #pragma unroll
     for (int i = 0; i < kOwn; ++i) {
       if (i * kThreads >= ns) break;
@@ -894,7 +895,9 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
         if (e16[i] >= kLobeMark) e16[i] = lobe[e16[i] & 63u];
       } else {
         e16[i] = ld_range(d.sel.hb + h0 + hbi[i]);
-        mx[i] = s.M[tid + i * kThreads];
+        far[i] = tid + i * kThreads < ns && !((unsigned)(sby[i] - nby) < (unsigned)nb &&
+                                              (unsigned)(sbx[i] - nbx) < (unsigned)nb);
+        if (far[i]) mx[i] = s.M[tid + i * kThreads];
       }
     }
     float pv[kCandPer];
@@ -919,8 +922,7 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
         acc[i].x = __fmaf_ru(m, __uint_as_float(w << 16), acc[i].x);
         acc[i].y = __fmaf_ru(m, __uint_as_float(w & 0xffff0000u), acc[i].y);
         bound = fmaxf(bound, fmaxf(acc[i].x, acc[i].y));
-      } else if (b < ns &&
-                 !((unsigned)(sby[i] - nby) < (unsigned)nb && (unsigned)(sbx[i] - nbx) < (unsigned)nb)) {
+      } else if (far[i]) {
         acc[i].x = __fmaf_ru(m, __uint_as_float(w << 16), acc[i].x);
         acc[i].y = __fmaf_ru(m, __uint_as_float(w & 0xffff0000u), acc[i].y);
         s.acc[b] = acc[i];

@@ -123,6 +123,7 @@ def test_first_candidates(emulator, tmp_path):
     (64, 64, (128, 128), 90, 1, 64),     # cells kept singly; more than one selection
     (61, 45, (61, 45), 30, 2, 64),       # a group of two, a clipped PSF, ragged cells
     (40, 56, (81, 113), 70, 3, 128),
+    (16, 17000, (32, 34000), 70, 2, 256),  # superblocks
 ])
 def test_no_races_and_the_oracles_bits(emulator, tmp_path, ny, nx, ps, niter, G, threads):
     dirty, psf = _field(ny, nx, ps, ny)
