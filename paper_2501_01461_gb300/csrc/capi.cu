@@ -245,7 +245,22 @@ int check_psf(clean_plan_s* pl, cudaStream_t s) {
   if (e == cudaSuccess) e = launch_validate_psf(pl->d, s);
   ++pl->kernel_launches;
   if (e != cudaSuccess) return cuda_fail(pl, e);
-  int rc = read_state(pl, s);
+  // what runs need of the PSF goes ahead of the status read (a PSF that fails
+  // the check is never run with), so that none of it is on its way when this
+  // returns: the next run may be on another stream
+  int rc = fft_prepare_psf(pl, s);
+  if (rc != CLEAN_OK) return rc;
+  if (pl->sel_ok) {
+    // cells past a tile's edge (row padding, smaller tiles) stay NaN: no bound
+    if (!pl->psf_set)
+      e = cudaMemsetAsync(pl->d.sel.u, 0xff,
+                          sizeof(float2) * (size_t)pl->d.sel.cell_stride * pl->d.T, s);
+    if (e == cudaSuccess)
+      e = select_build_psf(pl->d, pl->sel_boxes, pl->sel_h8, pl->sel_hb, pl->sel_lobe, s);
+    pl->kernel_launches += 4;
+    if (e != cudaSuccess) return cuda_fail(pl, e);
+  }
+  rc = read_state(pl, s);
   if (rc != CLEAN_OK) return rc;
   const int bits = pl->h_st.status;
   pl->psf_set = true;
@@ -253,12 +268,6 @@ int check_psf(clean_plan_s* pl, cudaStream_t s) {
                    : (bits & ST_PSF_OFFCENTRE) ? CLEAN_ERR_INVALID_ARG
                                                : CLEAN_OK;
   pl->started = false;  // a run's state refers to the old PSF
-  if (pl->psf_status == CLEAN_OK && (rc = fft_prepare_psf(pl, s)) != CLEAN_OK) return rc;
-  if (pl->psf_status == CLEAN_OK && pl->sel_ok) {
-    e = select_build_psf(pl->d, pl->sel_boxes, pl->sel_h8, pl->sel_hb, pl->sel_lobe, s);
-    pl->kernel_launches += 4;
-    if (e != cudaSuccess) return cuda_fail(pl, e);
-  }
   return pl->psf_status;
 }
 
@@ -901,9 +910,7 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
     clean_destroy(pl);
     return CLEAN_ERR_CUDA;
   }
-  // cells past a tile's edge (row padding, smaller tiles) stay NaN: no bound
-  if ((pl->sel_ok && cudaMemsetAsync(d.sel.u, 0xff, sel_z.cells, s) != cudaSuccess) ||
-      cudaMemsetAsync(d.gbar, 0, sizeof(uint32_t) * T, s) != cudaSuccess ||
+  if (cudaMemsetAsync(d.gbar, 0, sizeof(uint32_t) * T, s) != cudaSuccess ||
       cudaMemsetAsync(d.st, 0, sizeof(DevState), s) != cudaSuccess) {
     cudaGetLastError();
     clean_destroy(pl);
