@@ -8,7 +8,6 @@
 #include <cmath>
 
 #include "cleangb_internal.cuh"
-#include "ptx.cuh"
 
 namespace cleangb {
 
@@ -16,7 +15,9 @@ namespace {
 
 // Set-up: a warp a row, four pixels of a lane in flight.  Small images are
 // bound by the latency of a block's few loads (320 x 320 in four tiles: 12 us
-// with 16 rows a block one after another, now 5), large ones by memory.
+// with 16 rows a block one after another, now 5), large ones by memory.  The
+// dirty image may be the residual itself (host buffers, runs in place), so its
+// loads are ordinary ones: the compiler keeps them ahead of the stores.
 constexpr int kInitThreads = 256;
 constexpr int kInitRows = kInitThreads / 32;  // tile rows per init block
 
@@ -50,7 +51,7 @@ __global__ void __launch_bounds__(kInitThreads)
       float v[U];
 #pragma unroll
       for (int j = 0; j < U; ++j)
-        v[j] = c + 32 * j < W ? ptx::ld_nc(dirty + row + c + 32 * j) : 0.f;
+        v[j] = c + 32 * j < W ? dirty[row + c + 32 * j] : 0.f;
 #pragma unroll
       for (int j = 0; j < U; ++j) {
         if (c + 32 * j >= W) break;
