@@ -1038,8 +1038,8 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
     }
     if (fail) break;
   }
-  if (tid == 0) d.sel.ctl[t].near = near;
   __syncthreads();
+  if (tid == 0) d.sel.ctl[t].near = near;  // (every thread has read it)
   // the records, here and not an iteration at a time (the thread that kept them
   // came to every barrier some 500 cycles after the others): the list, and the
   // model, whose pixels' sums are taken in list order by the thread of the

@@ -105,7 +105,7 @@ def _check(emulator, tmp_path, dirty, psf, niter, thr=0.0, tiles=(1, 1), G=1, th
     o = oracle.clean_f32(dirty, psf, gain, niter, thr, tiles, 0)
     r, m, c = _emulate(emulator(threads), tmp_path, dirty, psf, gain, niter, thr, tiles, G)
     for k in ("y", "x", "tile"):
-        assert np.array_equal(c[k], o.comps[k]), k
+        assert np.array_equal(c[k], o.comps[k]), (k, c[k], o.comps[k])
     assert np.array_equal(c["flux"].view(np.uint32), o.comps["flux"].view(np.uint32))
     assert np.array_equal(r.view(np.uint32), o.residual.view(np.uint32))
     assert np.array_equal(m.view(np.uint32), o.model.view(np.uint32))
@@ -128,3 +128,12 @@ def test_first_candidates(emulator, tmp_path):
 def test_no_races_and_the_oracles_bits(emulator, tmp_path, ny, nx, ps, niter, G, threads):
     dirty, psf = _field(ny, nx, ps, ny)
     _check(emulator, tmp_path, dirty, psf, niter, G=G, threads=threads)
+
+
+def test_more_ties_than_candidates(emulator, tmp_path):
+    """One component a selection: it ends before its first barrier between
+    reading the tile's margin and writing it."""
+    psf = np.zeros((200, 220), np.float32)
+    psf[100, 110] = 1.0
+    dirty = synth.tie_image(100, 110, np.random.default_rng(3))
+    _check(emulator, tmp_path, dirty, psf, 20, tiles=(1, 2), gain=0.5)
