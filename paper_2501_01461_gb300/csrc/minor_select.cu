@@ -665,6 +665,7 @@ __device__ __forceinline__ int resolve(const PlanDev& d, const Geo& g, int n, fl
     if (add == 0) continue;
     slot = __shfl_sync(0xffffffffu, slot, 0);
     if (slot + add > kCand) continue;  // the selection ends
+    __syncwarp();  // every lane has read the mask
     if (lane == 0) __stcg(&g.masks[c], now);
     const uint32_t below = (1u << lane) - 1u;
     if ((n0 >> lane) & 1u) {

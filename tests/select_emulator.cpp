@@ -96,6 +96,16 @@ static void exchange(unsigned mask, uint32_t v, uint32_t (&all)[32]) {
   for (int i = 0; i < 32; ++i) all[i] = slot[i];
   if (AnnotateIgnoreSyncEnd) AnnotateIgnoreSyncEnd(__FILE__, __LINE__);
 }
+static void __syncwarp() {  // (one that does order memory)
+  Warp& w = cta->warps[threadIdx.x >> 5];
+  const int g = w.gen.load();
+  if (w.arrived.fetch_add(1) == 31) {
+    w.arrived = 0;
+    ++w.gen;
+  } else {
+    while (w.gen.load() == g) sched_yield();
+  }
+}
 template <class To, class From>
 static To bits(From v) {
   static_assert(sizeof(To) == sizeof(From), "");

@@ -137,3 +137,8 @@ def test_more_ties_than_candidates(emulator, tmp_path):
     psf[100, 110] = 1.0
     dirty = synth.tie_image(100, 110, np.random.default_rng(3))
     _check(emulator, tmp_path, dirty, psf, 20, tiles=(1, 2), gain=0.5)
+
+
+def test_resolved_cells_that_add_candidates(emulator, tmp_path):
+    rng = np.random.default_rng(5)
+    _check(emulator, tmp_path, synth.random_image(64, 48, rng), synth.random_psf(60, 50, rng), 150)
