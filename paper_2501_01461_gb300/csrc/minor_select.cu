@@ -96,10 +96,11 @@ __device__ __forceinline__ int ord(float v) {
   const int b = __float_as_int(v);
   return b ^ ((b >> 31) & 0x7fffffff);
 }
-__device__ __forceinline__ float warp_max_f(float v) {
+__device__ __forceinline__ float warp_max_f(float v) {  // (no NaN)
   const int o = __reduce_max_sync(0xffffffffu, ord(v));
   return __int_as_float(o ^ ((o >> 31) & 0x7fffffff));
 }
+// (a NaN, as an overflow leaves on a pixel, is no bound: the other value)
 __device__ __forceinline__ float2 max2(float2 a, float2 b) {
   return make_float2(fmaxf(a.x, b.x), fmaxf(a.y, b.y));
 }
@@ -566,7 +567,7 @@ __device__ __forceinline__ void start_candidates(const PlanDev& d, const Geo& g,
     const uint32_t h0 = __ballot_sync(0xffffffffu, c0), h1 = __ballot_sync(0xffffffffu, c1);
     if ((h0 | h1) == 0u) continue;  // as the pass left it
     float2 u = make_float2(-INFINITY, -INFINITY);
-    if (in0 && !c0) u = make_float2(v0, -v0);
+    if (in0 && !c0) u = max2(u, make_float2(v0, -v0));
     if (in1 && !c1) u = max2(u, make_float2(v1, -v1));
     u = make_float2(warp_max_f(u.x), warp_max_f(u.y));
     int slot = 0;
@@ -645,7 +646,7 @@ __device__ __forceinline__ int resolve(const PlanDev& d, const Geo& g, int n, fl
     const uint32_t n1 = __ballot_sync(0xffffffffu, in[1] && fabsf(r[1]) >= near) & ~was.y;
     const uint2 now = make_uint2(was.x | n0, was.y | n1);
     float2 u = make_float2(-INFINITY, -INFINITY);
-    if (in[0] && !((now.x >> lane) & 1u)) u = make_float2(r[0], -r[0]);
+    if (in[0] && !((now.x >> lane) & 1u)) u = max2(u, make_float2(r[0], -r[0]));
     if (in[1] && !((now.y >> lane) & 1u)) u = max2(u, make_float2(r[1], -r[1]));
     u = make_float2(warp_max_f(u.x), warp_max_f(u.y));
     const int add = __popc(n0) + __popc(n1);

@@ -142,3 +142,13 @@ def test_more_ties_than_candidates(emulator, tmp_path):
 def test_resolved_cells_that_add_candidates(emulator, tmp_path):
     rng = np.random.default_rng(5)
     _check(emulator, tmp_path, synth.random_image(64, 48, rng), synth.random_psf(60, 50, rng), 150)
+
+
+def test_cells_with_nan_pixels(emulator, tmp_path):
+    """A PSF that makes the residual overflow, and no wider than 3 pixels: some
+    pixels of a cell turn NaN, and its others still rise to the peak."""
+    dirty = synth.random_image(64, 64, np.random.default_rng(1), 1e-2)
+    dirty[10, 62], dirty[13, 61] = 3e38, 5.0
+    psf = np.zeros((3, 3), np.float32)
+    psf[1, 1] = psf[1, 2] = 400.0
+    _check(emulator, tmp_path, dirty, psf, 12)
