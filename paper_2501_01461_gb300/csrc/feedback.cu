@@ -195,7 +195,9 @@ __device__ __forceinline__ void feedback_body(const PlanDev& d, int parity, int 
 
 __global__ void __launch_bounds__(kThreads)
     feedback_kernel(PlanDev d, int parity, int apply, int blocks_x, int blocks_y) {
-  feedback_body(d, parity, apply, blockIdx.z, blockIdx.x, blockIdx.y, blocks_x, blocks_y);
+  // a tile's blocks along x: 16-row blocks of a tall image pass the 65,535 of y
+  feedback_body(d, parity, apply, blockIdx.y, blockIdx.x % blocks_x, blockIdx.x / blocks_x,
+                blocks_x, blocks_y);
 }
 
 
@@ -490,7 +492,7 @@ cudaError_t launch_feedback(const PlanDev& d, const CUtensorMap* psf_map, int pa
   }
   const int bx = (maxW + kCols - 1) / kCols, by = (maxH + kRows - 1) / kRows;
   const size_t smem = sizeof(Comp4) * kChunk + sizeof(int32_t) * (2 * (size_t)d.T + 1);
-  feedback_kernel<<<dim3(bx, by, d.T), kThreads, smem, s>>>(d, parity, apply, bx, by);
+  feedback_kernel<<<dim3(bx * by, d.T), kThreads, smem, s>>>(d, parity, apply, bx, by);
   return cudaGetLastError();
 }
 
