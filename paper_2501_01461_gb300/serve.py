@@ -53,16 +53,17 @@ def footprint_bytes(n: int, psf_shape, niter: int, tiles=(1, 1), K: int = 0,
                     feedback_mode: int = FB_GATHER) -> int:
     """Device bytes a job holds while resident: residual and model images,
     its PSF (held by the caller but pinned for the job's lifetime), the
-    component list and the round buffer, the minor loop's tables, and with FFT feedback the kernel
-    spectrum, the transforms' work areas and the round-start residual."""
+    component list and the round buffer, the minor loop's tables, and with FFT
+    feedback the kernel spectrum, the transforms' work areas and the round-start residual."""
     T = tiles[0] * tiles[1]
     per_tile = niter // T + (1 if niter % T else 0)
     cap = min(K, per_tile) if K > 0 else per_tile
     b = (8 * n * n + 4 * psf_shape[0] * psf_shape[1] + 16 * niter + 16 * T * max(cap, 1)
          + 8 * niter + 4096)
     # the minor loop's cells (bounds and candidate masks) and PSF ranges
-    m = -(-n // min(tiles))
-    b += 16 * T * (-(-m // 8) + 1) ** 2 + 24 * (2 * -(-m // 8) + 2) ** 2 + 16384
+    cy, cx = (-(-n // (8 * t)) for t in tiles)
+    b += 16 * T * cy * (cx + cx % 2) + 64 * T + 16384
+    b += (24 if cy * cx > 4096 else 12) * (2 * cy + 2) * (2 * cx + 2)
     if feedback_mode == FB_FFT and T > 1:
         L = _fft_size(2 * n - 1)
         # kernel spectrum, the round's column work area, the component list,

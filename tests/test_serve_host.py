@@ -26,3 +26,19 @@ def test_fifo_latencies():
     assert np.allclose(lat, [2.0, 2.0, 2.5])
     # unsorted input is served in arrival order
     assert np.allclose(sorted(serve.fifo_latencies([1.0, 0.0], [1.0, 1.0])), [1.0, 1.0])
+
+
+def test_footprint_counts_the_tables_of_the_tiles_there_are():
+    """Tile grids that are not square: the minor loop's cells and PSF tables
+    are those of the image's own tiles (a 64 x 1 grid of 4096 has 64 x 512
+    cells of 8 x 8 pixels a side, not 512 x 512 a tile)."""
+    for n, tiles in ((4096, (1, 64)), (4096, (64, 1)), (1000, (2, 3)), (300, (1, 1))):
+        T = tiles[0] * tiles[1]
+        cy, cx = (-(-n // (8 * t)) for t in tiles)
+        big = cy * cx > 4096
+        tables = (16 * T * cy * (cx + cx % 2)
+                  + (2 if big else 1) * (8 * (2 * cy + 2) * (2 * cx + 2)
+                                         + 4 * (2 * cy + 1) * (2 * cx + 1)))
+        images = 8 * n * n + 4 * 4 * n * n
+        f = serve.footprint_bytes(n, (2 * n, 2 * n), 1000, tiles, 50)
+        assert images + tables <= f <= images + tables + (1 << 18), (n, tiles, f, tables)
