@@ -119,9 +119,10 @@ def candidates(tiles, sm_count: int, allow_fft: bool = False) -> list[Choice]:
         if G * T <= 4 * sm_count:
             out.append(Choice(group_ctas=G, group_sync=SYNC_CLUSTER))
     out.append(Choice(feedback_path=1))
-    # the automatic minor loop without tile pairs, and without TMEM chunks
-    out.append(Choice(minor_pairs=0))
-    out.append(Choice(minor_tmem=0))
+    # the bulk-copy pipeline on the library's groups without tile pairs, and without
+    # TMEM chunks (the automatic minor loop, by selection, has neither)
+    out.append(Choice(minor_path=2, minor_pairs=0))
+    out.append(Choice(minor_path=2, minor_tmem=0))
     if allow_fft and T > 1:
         out.append(Choice(feedback_mode=FB_FFT))
     # keep order, drop duplicates

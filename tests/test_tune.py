@@ -87,3 +87,13 @@ def test_tuned_interval_stays_in_paper_band():
     for t in res.k_trials:
         assert t["in_band"] == (tune.PAPER_BAND[0] <= t["min_diff"] and
                                 t["max_diff"] <= tune.PAPER_BAND[1])
+
+
+def test_candidates_without_pairs_or_tmem_do_not_run_by_selection():
+    """Pairs and tensor-memory chunks belong to the bulk-copy pipeline; with the
+    group, the barrier and the path left to the library a plan selects, and two
+    such candidates would time one kernel."""
+    for tiles in ((1, 1), (2, 2), (4, 4)):
+        for c in tune.candidates(tiles, 152):
+            if not c.minor_pairs or not c.minor_tmem:
+                assert c.minor_path == 2 or c.group_ctas or c.group_sync != cg.SYNC_AUTO, c
