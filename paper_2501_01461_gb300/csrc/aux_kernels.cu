@@ -114,52 +114,70 @@ __global__ void validate_psf_kernel(const float* __restrict__ P, int64_t n, int6
 // Restore: out[q] = R[q] + sum over offsets o in the disc |o| <= r of
 // model[q - o] * B(o), B the clean beam (symmetric, so B(o) = B(-o)).
 //
-// A model is components on few pixels, so a block of output pixels lists the
-// non-zero model pixels that reach it and adds only their beams, in the order
-// of the full sum (descending rows, then columns): the skipped terms are zeros,
-// and the sums are those of the full convolution bit for bit.  Bound by reading
-// the model window (64 + 2 r)^2 a block and listing its pixels: 0.079 ms at
-// 2048^2 with r = 28 and 8000 components, 3.03 ms with the full sum.
-constexpr int kRB = 64;              // output block side
-constexpr int kRThreads = 512;
-constexpr int kRRows = kRB * kRB / kRThreads;  // output rows a thread sums
-constexpr int kRList = 2048;         // window pixels looked at in one go
-constexpr int kRPer = kRList / kRThreads;
+// A CLEAN model is components on few pixels, so a block of output pixels goes
+// through the model window that reaches it some rows at a time, from the last
+// row and column backwards, and either lists those rows' non-zero pixels and
+// adds their beams or, when they are many, sums the rows whole.  Both add a
+// pixel's terms in the order of the full sum (descending rows, then columns);
+// the terms left out are zeros, so the sums are those of the full convolution
+// bit for bit.  Bound by reading the window while sources are few (2048^2, r 28:
+// 0.098 ms at 0.2 % of the pixels, 2.97 with every sum whole), by the taps of the
+// rows summed whole when they are many (2.2 ms at 40 to 100 %, 0.31 to 0.18 at
+// 256^2; a kernel of lists alone took 14.2 and 3.2 there, one of full sums 2.97
+// and 0.31).
+constexpr int kRList = 2048;         // window pixels looked at in one go, whole rows
 constexpr int kRCounts = kRList / 32;
+// a listed pixel costs about what kRDense taps of a row summed whole cost (between
+// 4 and 6 nothing is slower than the full sum at any density, r 12 to 59, 100^2 to
+// 2048^2; at 3 lists were, by up to 15 % at 20 %)
+constexpr int kRDense = 5;
 
-__global__ void __launch_bounds__(kRThreads)
+// images below this many pixels: smaller blocks, to fill the SMs (256^2, r 12, 10 %:
+// 0.07 ms, 0.2 with the larger ones; 2048^2, r 59, 0.2 %: 0.19 with those, 0.37)
+constexpr int64_t kRSmallPx = 1 << 20;
+
+// RB x RB output pixels, ROWS of a column to a thread
+template <int RB, int ROWS>
+__global__ void __launch_bounds__(RB * RB / ROWS, 1024 * ROWS / (RB * RB))
     restore_kernel(PlanDev d, const float* __restrict__ beam, int r, float* __restrict__ out) {
+  constexpr int kThreads = RB * RB / ROWS, kWarps = kThreads / 32, kPer = kRList / kThreads;
   extern __shared__ __align__(16) float sm[];
-  int4* s_src = reinterpret_cast<int4*>(sm);         // row, column, value of each source
+  int4* s_src = reinterpret_cast<int4*>(sm);         // row, column, value of each source,
+  float* s_rows = sm;                                // or the rows
   float* s_beam = sm + 4 * kRList;                   // (2r+1)^2
   __shared__ int s_first[kRCounts + 1];              // sources before each warp's 32 pixels
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int y0 = blockIdx.y * kRB, x0 = blockIdx.x * kRB;
-  const int n = 2 * r + 1, side = kRB + 2 * r;
-  const int x = x0 + threadIdx.x % kRB, yt = y0 + threadIdx.x / kRB;
-  constexpr int kStep = kRThreads / kRB;             // a thread's rows: yt, yt + kStep, ...
-  for (int i = threadIdx.x; i < n * n; i += kRThreads) s_beam[i] = beam[i];
-  float acc[kRRows];
+  const int n = 2 * r + 1, side = RB + 2 * r, most = kRList / side;
+  const int y0 = blockIdx.y * RB, x0 = blockIdx.x * RB;
+  const int ylast = y0 + RB - 1 + r, xlast = x0 + RB - 1 + r;
+  const int tx = threadIdx.x % RB, ty = threadIdx.x / RB * ROWS;
+  for (int i = threadIdx.x; i < n * n; i += kThreads) s_beam[i] = beam[i];
+  float acc[ROWS];
 #pragma unroll
-  for (int k = 0; k < kRRows; ++k) acc[k] = 0.f;
+  for (int k = 0; k < ROWS; ++k) acc[k] = 0.f;
+  int pr[kPer], pc[kPer];  // the thread's pixels of the rows
+#pragma unroll
+  for (int k = 0; k < kPer; ++k) {
+    const int i = k * kThreads + (int)threadIdx.x;
+    pr[k] = i / side;
+    pc[k] = i - pr[k] * side;
+  }
 
-  const int total = side * side;
-  for (int i0 = 0; i0 < total; i0 += kRList) {
-    // pixel i of the window, from its last row and column backwards
-    float v[kRPer];
-    uint32_t nz[kRPer];
+  for (int w0 = 0; w0 < side; w0 += most) {
+    const int rows = min(most, side - w0);
+    float v[kPer];
+    uint32_t nz[kPer];
 #pragma unroll
-    for (int k = 0; k < kRPer; ++k) {
-      const int i = i0 + k * kRThreads + (int)threadIdx.x;
-      const int yy = y0 + kRB - 1 + r - i / side, xx = x0 + kRB - 1 + r - i % side;
-      v[k] = i < total && yy >= 0 && yy < d.ny && xx >= 0 && xx < d.nx
+    for (int k = 0; k < kPer; ++k) {
+      const int yy = ylast - w0 - pr[k], xx = xlast - pc[k];
+      v[k] = pr[k] < rows && yy >= 0 && yy < d.ny && xx >= 0 && xx < d.nx
                  ? d.model[(int64_t)yy * d.nx + xx] : 0.f;
     }
-    __syncthreads();  // the last list has been used
+    __syncthreads();  // the last rows have been used
 #pragma unroll
-    for (int k = 0; k < kRPer; ++k) {
+    for (int k = 0; k < kPer; ++k) {
       nz[k] = __ballot_sync(0xffffffffu, v[k] != 0.f);
-      if (lane == 0) s_first[k * (kRThreads / 32) + warp] = __popc(nz[k]);
+      if (lane == 0) s_first[k * kWarps + warp] = __popc(nz[k]);
     }
     __syncthreads();
     if (warp == 0) {  // exclusive prefix of the counts
@@ -180,33 +198,66 @@ __global__ void __launch_bounds__(kRThreads)
     __syncthreads();
     const int ns = s_first[kRCounts];
     if (ns == 0) continue;  // the same for the whole block
+    // the image's rows among them
+    const int j0 = max(ylast - w0 - (d.ny - 1), 0), j1 = min(ylast - w0 + 1, rows);
+    const bool whole = ns * kRDense > (j1 - j0) * n;
 #pragma unroll
-    for (int k = 0; k < kRPer; ++k)
-      if (v[k] != 0.f) {
-        const int i = i0 + k * kRThreads + (int)threadIdx.x;
-        const int at = s_first[k * (kRThreads / 32) + warp] + __popc(nz[k] & ((1u << lane) - 1u));
-        s_src[at] = make_int4(y0 + kRB - 1 + r - i / side, x0 + kRB - 1 + r - i % side,
-                              __float_as_int(v[k]), 0);
+    for (int k = 0; k < kPer; ++k) {
+      if (whole) {
+        if (pr[k] < rows) s_rows[k * kThreads + threadIdx.x] = v[k];
+      } else if (v[k] != 0.f) {
+        const int at = s_first[k * kWarps + warp] + __popc(nz[k] & ((1u << lane) - 1u));
+        s_src[at] = make_int4(ylast - w0 - pr[k], xlast - pc[k], __float_as_int(v[k]), 0);
       }
+    }
     __syncthreads();
-    for (int j = 0; j < ns; ++j) {
-      const int4 c = s_src[j];
-      const int ox = x - c.y + r, oy = yt - c.x + r;
-      if ((unsigned)ox >= (unsigned)n) continue;
-      const float m = __int_as_float(c.z);
+    if (whole) {
+      for (int j = j0; j < j1; ++j) {
+        const int oy = y0 + ty - (ylast - w0 - j) + r;  // the first row's; a warp's own
+        if (oy + ROWS <= 0 || oy >= n) continue;
+        const float* m = s_rows + j * side + RB - 1 - tx;
+        const float* bp = s_beam + oy * n;
+        if (oy >= 0 && oy + ROWS <= n) {
+#pragma unroll 2
+          for (int o = 0; o < n; ++o) {
+            const float mv = m[o];
 #pragma unroll
-      for (int k = 0; k < kRRows; ++k) {
-        const int o = oy + k * kStep;
-        if ((unsigned)o < (unsigned)n) {
-          const float b = s_beam[o * n + ox];
-          if (b != 0.f) acc[k] = fmaf(m, b, acc[k]);
+            for (int k = 0; k < ROWS; ++k) {
+              const float b = bp[k * n + o];
+              if (b != 0.f) acc[k] = fmaf(mv, b, acc[k]);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < ROWS; ++k) {
+            if ((unsigned)(oy + k) >= (unsigned)n) continue;
+#pragma unroll 4
+            for (int o = 0; o < n; ++o) {
+              const float b = bp[k * n + o];
+              if (b != 0.f) acc[k] = fmaf(m[o], b, acc[k]);
+            }
+          }
+        }
+      }
+    } else {
+      for (int j = 0; j < ns; ++j) {
+        const int4 c = s_src[j];
+        const int oy = y0 + ty - c.x + r, ox = x0 + tx - c.y + r;
+        if (oy + ROWS <= 0 || oy >= n || (unsigned)ox >= (unsigned)n) continue;
+        const float m = __int_as_float(c.z);
+#pragma unroll
+        for (int k = 0; k < ROWS; ++k) {
+          if ((unsigned)(oy + k) < (unsigned)n) {
+            const float b = s_beam[(oy + k) * n + ox];
+            if (b != 0.f) acc[k] = fmaf(m, b, acc[k]);
+          }
         }
       }
     }
   }
 #pragma unroll
-  for (int k = 0; k < kRRows; ++k) {
-    const int y = yt + k * kStep;
+  for (int k = 0; k < ROWS; ++k) {
+    const int y = y0 + ty + k, x = x0 + tx;
     if (y < d.ny && x < d.nx)
       out[(int64_t)y * d.nx + x] = d.R[(int64_t)y * d.nx + x] + acc[k];
   }
@@ -275,11 +326,15 @@ cudaError_t launch_restore_with(const PlanDev& d, float bmaj, float bmin, float 
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   const size_t smem = sizeof(int4) * kRList + sizeof(float) * (size_t)(2 * r + 1) * (2 * r + 1);
-  e = allow_max_smem((const void*)restore_kernel);
-  if (e != cudaSuccess) return e;
-  dim3 grid((d.nx + kRB - 1) / kRB, (d.ny + kRB - 1) / kRB, 1);
-  restore_kernel<<<grid, kRThreads, smem, s>>>(d, beam_buf, r, out);
-  return cudaGetLastError();
+  auto launch = [&](auto kernel, int side, int threads) {
+    const cudaError_t err = allow_max_smem((const void*)kernel);
+    if (err != cudaSuccess) return err;
+    const dim3 grid((d.nx + side - 1) / side, (d.ny + side - 1) / side, 1);
+    kernel<<<grid, threads, smem, s>>>(d, beam_buf, r, out);
+    return cudaGetLastError();
+  };
+  if ((int64_t)d.ny * d.nx < kRSmallPx) return launch(restore_kernel<32, 4>, 32, 256);
+  return launch(restore_kernel<64, 8>, 64, 512);
 }
 
 }  // namespace cleangb
