@@ -126,7 +126,9 @@ typedef struct {
   int64_t n_components;   /* components in the list */
   int64_t rounds;         /* rounds that produced at least one component */
   int64_t rounds_launched;/* rounds launched, including no-op rounds */
-  int32_t group_ctas;     /* CTAs per tile chosen for the minor loop */
+  /* the iteration-by-iteration minor loop's launch, group_ctas to minor_pairs;
+     clean_minor_info tells whether the run's rounds go by selection instead */
+  int32_t group_ctas;     /* CTAs per tile */
   int32_t group_sync;     /* CLEAN_SYNC_CLUSTER or CLEAN_SYNC_GRID */
   int32_t resident;       /* 1 if each CTA keeps its residual rows in shared memory */
   int32_t feedback_mode;  /* the feedback path in use */
@@ -391,6 +393,15 @@ CLEAN_API int clean_probe_l2_read(const void* d_buf, int64_t bytes, int32_t pass
                                   float* ms, void* stream);
 
 /* Fills *out (host) with the plan's counters.  Synchronises. */
+/* The minor loop that a plan's rounds launch: *by_selection 1 for selection
+ * (*ctas CTAs per tile), 0 for the iteration-by-iteration loop (as clean_stats
+ * describes it).  *taken_over: how many times in the current run that loop has
+ * taken the rest of a tile's round over from the selection, where it is the
+ * faster (crowded fields deep in their noise).  Any output may be NULL.
+ * Synchronises. */
+CLEAN_API int clean_minor_info(clean_plan_t plan, int32_t* by_selection, int32_t* ctas,
+                               int64_t* taken_over, void* stream);
+
 CLEAN_API int clean_stats(clean_plan_t plan, clean_stats_t* out, void* stream);
 
 /* Frees everything the plan owns (not the borrowed PSF).  NULL is a no-op.
@@ -417,9 +428,7 @@ CLEAN_API const char* clean_strerror(int status);
  *                              Same results, bit for bit.
  *   CLEAN_DEBUG_MINOR_PATH     minor-loop kernel: 0 automatic (selection when
  *                              group_ctas and group_sync are left to the
- *                              library and no tile side is above 32767, but
- *                              for one small tile run without a threshold far
- *                              into its noise; else
+ *                              library and no tile side is above 32767; else
  *                              the bulk-copy pipeline when image and PSF rows
  *                              are 16-byte aligned), 1 plain loads, 2 pipeline
  *                              when possible (same results, bit for bit)
@@ -441,6 +450,14 @@ CLEAN_API const char* clean_strerror(int status);
  *                              exchange overlaps the other's pass
  *                              (clean_stats_t.minor_pairs); 0: a group per
  *                              tile.  Same results, bit for bit.
+ *   CLEAN_DEBUG_PLAIN_CYCLES   SM cycles that an iteration of the plain loop is
+ *                              taken to cost (a tile whose selections cost more
+ *                              is handed over to it; 0: none is);
+ *                              CLEAN_ERR_INVALID_ARG where the plan has no such
+ *                              launch (several tiles with rounds of up to 64
+ *                              iterations or a flux trigger, or tiles too large
+ *                              for its groups' shared memory).  Same results,
+ *                              bit for bit.
  *   CLEAN_DEBUG_TIMING         1: bracket every minor-loop and feedback launch
  *                              with CUDA events on its stream and sum their
  *                              durations into clean_stats (0: off, resets)
@@ -457,7 +474,8 @@ enum {
   CLEAN_DEBUG_PIPE_STAGES = 7,
   CLEAN_DEBUG_GRAPHS = 8,
   CLEAN_DEBUG_MINOR_TMEM = 9,
-  CLEAN_DEBUG_MINOR_PAIR = 10
+  CLEAN_DEBUG_MINOR_PAIR = 10,
+  CLEAN_DEBUG_PLAIN_CYCLES = 11
 };
 CLEAN_API int clean_debug_set(clean_plan_t plan, int32_t what, int64_t value);
 CLEAN_API void clean_debug_alloc_limit(int64_t bytes);

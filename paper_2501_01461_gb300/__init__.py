@@ -24,7 +24,7 @@ __all__ = ["CleanError", "Plan", "Batch", "lib", "library_path", "build", "STATU
            "SYNC_AUTO", "SYNC_CLUSTER", "SYNC_GRID", "COMPONENT_DTYPE",
            "DEBUG_SPIN_LIMIT_NS", "DEBUG_FORCE_TIMEOUT", "DEBUG_TIMING", "DEBUG_FEEDBACK_PATH", "DEBUG_MINOR_PATH",
            "DEBUG_PIPE_CHUNK_PX", "DEBUG_PIPE_STAGES", "DEBUG_GRAPHS", "DEBUG_MINOR_TMEM",
-           "DEBUG_MINOR_PAIR", "probe_l2_read",
+           "DEBUG_MINOR_PAIR", "DEBUG_PLAIN_CYCLES", "probe_l2_read",
            "EXPORTED_SYMBOLS"]
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
@@ -33,7 +33,7 @@ TILED, UNTILED_GRID = 0, 1
 SYNC_AUTO, SYNC_CLUSTER, SYNC_GRID = 0, 1, 2
 DEBUG_SPIN_LIMIT_NS, DEBUG_FORCE_TIMEOUT, DEBUG_TIMING = 1, 2, 3
 DEBUG_FEEDBACK_PATH, DEBUG_MINOR_PATH, DEBUG_PIPE_CHUNK_PX, DEBUG_PIPE_STAGES = 4, 5, 6, 7
-DEBUG_GRAPHS, DEBUG_MINOR_TMEM, DEBUG_MINOR_PAIR = 8, 9, 10
+DEBUG_GRAPHS, DEBUG_MINOR_TMEM, DEBUG_MINOR_PAIR, DEBUG_PLAIN_CYCLES = 8, 9, 10, 11
 STATUS = {0: "CLEAN_OK", 1: "CLEAN_ERR_INVALID_ARG", 2: "CLEAN_ERR_NONFINITE",
           3: "CLEAN_ERR_OOM", 4: "CLEAN_ERR_CUDA", 5: "CLEAN_ERR_TIMEOUT",
           6: "CLEAN_ERR_UNSUPPORTED"}
@@ -90,6 +90,7 @@ _SIGS = {
     "clean_checkpoint": (ctypes.c_int, [_vp, _vp, _i64, _vp, _vp]),
     "clean_resume": (ctypes.c_int, [_vp, _vp, _i64, _vp]),
     "clean_stats": (ctypes.c_int, [_vp, _vp, _vp]),
+    "clean_minor_info": (ctypes.c_int, [_vp, _vp, _vp, _vp, _vp]),
     "clean_destroy": (None, [_vp]),
     "clean_strerror": (ctypes.c_char_p, [ctypes.c_int]),
     "clean_debug_set": (ctypes.c_int, [_vp, _i32, _i64]),
@@ -328,6 +329,14 @@ class Plan:
         s = Stats()
         _check(lib().clean_stats(self._h, ctypes.byref(s), _stream_ptr(stream)), "clean_stats")
         return {f: getattr(s, f) for f, _ in Stats._fields_}
+
+    def minor_info(self, stream=None) -> dict:
+        """The minor loop that the rounds launch (see clean_minor_info)."""
+        sel, ctas, taken = ctypes.c_int32(0), ctypes.c_int32(0), ctypes.c_int64(0)
+        _check(lib().clean_minor_info(self._h, ctypes.byref(sel), ctypes.byref(ctas),
+                                      ctypes.byref(taken), _stream_ptr(stream)),
+               "clean_minor_info")
+        return dict(by_selection=bool(sel.value), ctas=ctas.value, taken_over=taken.value)
 
     def deconvolve_host(self, dirty: np.ndarray, psf: np.ndarray | None = None,
                         residual: np.ndarray | None = None, model: np.ndarray | None = None,

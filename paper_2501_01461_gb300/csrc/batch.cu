@@ -53,6 +53,7 @@ struct Group {
   int offset = 0, count = 0;  // into the item array
   int G = 1, smem = 0;
   int select = 0;             // 1: selection, 0: plain loads
+  int takeover = 0;           // plain loads for tiles that their selections handed over
   int direct = 0;             // selection without superblocks
   int resident = 0;           // plain loads: rows in shared memory
 };
@@ -204,6 +205,16 @@ void tile_group(int h, int w, int* G, int* resident, int* smem) {
   *smem = 0;
 }
 
+// The same for a launch that takes tiles over from their selections: where SMs
+// are idle (`most` a tile), more CTAs, down to 2048 pixels each.
+void takeover_group(int h, int w, int most, int* G, int* resident, int* smem) {
+  tile_group(h, w, G, resident, smem);
+  while (*resident && *G < 16 && 2 * *G <= std::min(most, h) && (int64_t)*G * 2048 < (int64_t)h * w) {
+    *G *= 2;
+    *smem = (h + *G - 1) / *G * w * 4;
+  }
+}
+
 // CTAs per tile of a selection.  With at most kSelPending iterations a round
 // the tile is scanned once and the rest is one CTA's; a round of several
 // selections passes over the tile between them, which a cluster shares (about
@@ -237,15 +248,20 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
   std::vector<BatchImage> imgs;
   struct Sized {
     int64_t px;
-    int select, direct, G, resident, smem;
+    int select, direct, G, resident, smem, takeover;
     BatchItem it;
   };
   std::vector<Sized> all;
   int block0 = 0;
   e->blocks_tma = e->blocks_plain = 0;
+  int sms = 0;
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->device);
+  int64_t n_tiles = 0;
+  for (int w : work) n_tiles += e->jobs[w].dev.T;
   for (int w = 0; w < (int)work.size(); ++w) {
     Job& j = e->jobs[work[w]];
     plans.push_back(j.dev);
+    plans.back().sel.plain_cycles = 0.f;  // (its own launches' value)
     maps.push_back(j.map);
     if (j.fft)
       e->fft_work.push_back(w);
@@ -254,6 +270,20 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
     if (j.tma && !j.fft) ++e->n_tma;
     e->max_T = std::max(e->max_T, j.dev.T);
     const int sel_G = j.sel_smem ? select_group(j.dev) : 0;
+    // behind the selections: the plain loop, for tiles on which it is the faster
+    // (see minor_select.cu); one group size for the image
+    Sized takeover{};
+    if (j.sel_smem && takeover_possible(j.dev)) {
+      const int h = (j.dev.ny + j.dev.ty - 1) / j.dev.ty, wd = (j.dev.nx + j.dev.tx - 1) / j.dev.tx;
+      takeover.takeover = 1;
+      takeover_group(h, wd, (int)(sms / n_tiles), &takeover.G, &takeover.resident, &takeover.smem);
+      if (takeover.resident) {
+        MinorCfg c{};
+        c.G = takeover.G;
+        c.sync = CLEAN_SYNC_CLUSTER;
+        plans.back().sel.plain_cycles = minor_plain_cycles(c, h, wd);
+      }
+    }
     for (int t = 0; t < j.dev.T; ++t) {
       const Rect r = tile_rect(t, j.dev.ny, j.dev.nx, j.dev.ty, j.dev.tx);
       Sized z{};
@@ -268,6 +298,12 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
       }
       z.it = BatchItem{w, t};
       all.push_back(z);
+      if (takeover.resident) {
+        Sized p = takeover;
+        p.px = z.px;
+        p.it = z.it;
+        all.push_back(p);
+      }
     }
     int bx = 0, by = 0;
     feedback_blocks(j.dev, j.tma, &bx, &by);
@@ -285,7 +321,7 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
   }
   // groups of one launch each, biggest tiles first within each
   auto kind = [](const Sized& z) {
-    return ((z.select * 2 + z.direct) * 2 + z.resident) * 32 + z.G;
+    return (((1 - z.takeover) * 2 + z.select) * 2 + z.direct) * 64 + z.resident * 32 + z.G;
   };
   std::stable_sort(all.begin(), all.end(), [&](const Sized& a, const Sized& b) {
     return kind(a) != kind(b) ? kind(a) > kind(b) : a.px > b.px;
@@ -300,6 +336,7 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
       g.direct = all[k].direct;
       g.G = all[k].G;
       g.resident = all[k].resident;
+      g.takeover = all[k].takeover;
       e->groups.push_back(g);
     }
     Group& g = e->groups.back();
@@ -307,11 +344,17 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
     ++g.count;
     items.push_back(all[k].it);
   }
-  for (const Group& g : e->groups)
+  for (size_t k = e->groups.size(); k-- > 0;) {
     // a cluster size the device cannot schedule
-    if (g.G > 1 && !(g.select ? select_cluster_fits(g.direct, g.G, g.smem)
+    const Group& g = e->groups[k];
+    if (g.G == 1 || (g.select ? select_cluster_fits(g.direct, g.G, g.smem)
                               : minor_batch_cluster(g.G, g.resident, g.smem) == g.G))
-      return CLEAN_ERR_UNSUPPORTED;
+      continue;
+    if (!g.takeover) return CLEAN_ERR_UNSUPPORTED;
+    for (int i = g.offset; i < g.offset + g.count; ++i)  // the selections take the whole rounds
+      plans[items[i].image].sel.plain_cycles = 0.f;
+    e->groups.erase(e->groups.begin() + (long)k);
+  }
   if ((int)items.size() > e->items_cap) {
     cudaFree(e->d_items);
     e->items_cap = std::max<int>((int)items.size(), 2 * e->items_cap);
@@ -387,7 +430,7 @@ cudaError_t launch_round(clean_engine_s* e, int round, cudaStream_t s, int* n) {
     err = g.select ? launch_select_batch(e->d_plans, e->d_items + g.offset, g.count, g.direct, g.G,
                                          g.smem, round, 2000000000ull, s)
                    : launch_minor_batch(e->d_plans, e->d_items + g.offset, g.count, g.G,
-                                        g.resident, g.smem, round, s);
+                                        g.resident, g.smem, g.takeover, round, s);
     ++*n;
     if (err != cudaSuccess) return err;
   }

@@ -97,7 +97,7 @@ struct clean_plan_s {
     PlanDev d;
     MinorCfg mc;
     CUtensorMap r_map, p_map, psf_map;
-    int32_t pipe, fb_path, tma, apply, select, sel_G, sel_smem;
+    int32_t pipe, fb_path, tma, apply, select, sel_G, sel_smem, takeover;
   };
   cudaStream_t cap_stream = nullptr;
   cudaGraphExec_t pair[2] = {nullptr, nullptr};
@@ -313,25 +313,27 @@ bool use_pipe(const clean_plan_s* pl) {
   return !pl->mc_pipe.resident;
 }
 
-bool deep_small(const clean_plan_s* pl) {
-  // one small tile cleaned far into its noise (no threshold, an iteration for
-  // every ten pixels): most cells come near the peak again and again there, and
-  // the plain loop's cluster takes 3.0 us an iteration whatever the image
-  // (256^2 with 250 sources: 3.1 against 4.6 by selection; with 20: 2.5)
-  const int64_t px = (int64_t)pl->p.ny * pl->p.nx;
-  return pl->d.T == 1 && px <= 65536 && !(pl->d.thr > 0.f) && !(pl->d.trigger > 0.f) &&
-         (pl->d.K <= 0 || pl->d.K > kSelPending) && pl->p.niter >= std::max<int64_t>(2000, px / 10);
-}
-
 // Selection whenever the caller left the tile groups and the minor-loop
 // variant to the library.
 bool use_select(const clean_plan_s* pl) {
-  return !deep_small(pl) && pl->sel_ok && pl->minor_path == 0 && pl->p.group_ctas == 0 &&
+  return pl->sel_ok && pl->minor_path == 0 && pl->p.group_ctas == 0 &&
          pl->p.group_sync == CLEAN_SYNC_AUTO;
+}
+
+// A launch of the plain loop behind the selection takes over the tiles on which
+// a selection turned out slower (minor_select.cu): crowded fields cleaned far
+// into their noise, where most cells come near the peak again and again.
+bool use_takeover(const clean_plan_s* pl) {
+  return use_select(pl) && pl->d.sel.plain_cycles > 0.f;
 }
 
 // flush: the residual must hold every component after the launch (a caller
 // may look at it before the feedback).
+MinorCfg takeover_cfg(MinorCfg c) {
+  c.takeover = 1;
+  return c;
+}
+
 int launch_round_minor(clean_plan_s* pl, cudaStream_t s, bool flush) {
   const bool pipe = use_pipe(pl);
   const int ev = timed_begin(pl, 0, s);
@@ -340,6 +342,10 @@ int launch_round_minor(clean_plan_s* pl, cudaStream_t s, bool flush) {
                                      (uint64_t)pl->mc.spin_limit_ns, pl->mc.force_timeout, s)
                      : launch_minor(pl->d, pipe ? pl->mc_pipe : pl->mc, pl->parity, &pl->r_map,
                                     &pl->p_map_minor, s);
+  if (e == cudaSuccess && use_takeover(pl)) {
+    e = launch_minor(pl->d, takeover_cfg(pl->mc), pl->parity, nullptr, nullptr, s);
+    ++pl->kernel_launches;
+  }
   timed_end(pl, ev, s);
   ++pl->kernel_launches;
   if (e != cudaSuccess) return cuda_fail(pl, e);
@@ -373,6 +379,7 @@ clean_plan_s::GraphKey graph_key(const clean_plan_s* pl) {
   k.select = use_select(pl) ? 1 : 0;
   k.sel_G = pl->sel_G;
   k.sel_smem = pl->sel_smem;
+  k.takeover = use_takeover(pl) ? 1 : 0;
   return k;
 }
 
@@ -382,6 +389,8 @@ cudaError_t launch_round_pair_part(const clean_plan_s* pl, const clean_plan_s::G
   cudaError_t e = k.select ? launch_select(k.d, k.sel_G, k.sel_smem, q, 0, (uint64_t)k.mc.spin_limit_ns,
                                            k.mc.force_timeout, s)
                            : launch_minor(k.d, k.mc, q, &k.r_map, &k.p_map, s);
+  if (e == cudaSuccess && k.takeover)
+    e = launch_minor(k.d, takeover_cfg(pl->mc), q, nullptr, nullptr, s);
   if (e != cudaSuccess) return e;
   return launch_feedback(k.d, k.tma ? &k.psf_map : nullptr, q, k.apply,
                          (uint64_t)pl->mc.spin_limit_ns, s);
@@ -434,7 +443,7 @@ int launch_pair(clean_plan_s* pl, cudaStream_t s) {
   }
   const cudaError_t e = cudaGraphLaunch(pl->pair[par], s);
   if (e != cudaSuccess) return cuda_fail(pl, e);
-  pl->kernel_launches += 4;
+  pl->kernel_launches += k.takeover ? 6 : 4;
   pl->rounds_launched += 2;
   ++pl->graph_launches;
   return CLEAN_OK;
@@ -903,6 +912,7 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
   d.sel.lobe = pl->sel_lobe;
   d.sel.inside = d.cy >= maxH - 1 && d.pny - d.cy >= maxH && d.cx >= maxW - 1 &&
                  d.pnx - d.cx >= maxW;
+  if (mc.resident && takeover_possible(d)) d.sel.plain_cycles = minor_plain_cycles(mc, maxH, maxW);
 
   if (pl->fft && (fft_make_twiddles(pl->fft_twy, pl->fft_ay, s) != cudaSuccess ||
                   fft_make_twiddles(pl->fft_twx, pl->fft_ax, s) != cudaSuccess)) {
@@ -1258,6 +1268,22 @@ int clean_stats(clean_plan_t pl, clean_stats_t* out, void* stream) {
   return CLEAN_OK;
 }
 
+int clean_minor_info(clean_plan_t pl, int32_t* by_selection, int32_t* ctas, int64_t* taken_over,
+                     void* stream) {
+  if (!pl) return CLEAN_ERR_INVALID_ARG;
+  if (pl->poisoned != CLEAN_OK) return pl->poisoned;
+  const bool sel = use_select(pl);
+  if (by_selection) *by_selection = sel ? 1 : 0;
+  if (ctas) *ctas = sel ? pl->sel_G : pl->mc.G;
+  if (!taken_over) return CLEAN_OK;
+  *taken_over = 0;
+  if (!pl->started) return CLEAN_OK;
+  DeviceGuard g(pl->device);
+  const int rc = read_state(pl, as_stream(stream));
+  if (rc == CLEAN_OK) *taken_over = pl->h_st.taken_over;
+  return rc;
+}
+
 int clean_debug_set(clean_plan_t pl, int32_t what, int64_t value) {
   if (!pl) return CLEAN_ERR_INVALID_ARG;
   switch (what) {
@@ -1345,6 +1371,11 @@ int clean_debug_set(clean_plan_t pl, int32_t what, int64_t value) {
       if (value < 0 || value > 1) return CLEAN_ERR_INVALID_ARG;
       pl->use_graphs = value != 0;
       pl->graphs_refused = false;
+      return CLEAN_OK;
+    case CLEAN_DEBUG_PLAIN_CYCLES:
+      if (value < 0 || value > (1 << 30) || !pl->mc.resident || !takeover_possible(pl->d))
+        return CLEAN_ERR_INVALID_ARG;
+      pl->d.sel.plain_cycles = (float)value;
       return CLEAN_OK;
     case CLEAN_DEBUG_TIMING:
       pl->timing = value != 0;

@@ -79,7 +79,7 @@ struct DevState {
   int64_t max_budget;    // max over tiles of the remaining budget
   int64_t timeout_where; // diagnostic: tile * 2^32 + barrier index of a timeout
   float level;           // flux-trigger level of the next round (0: none)
-  int32_t pad1;
+  int32_t taken_over;   // tiles' rounds that the plain loop took over from the selection
 };
 
 // Selection minor loop (minor_select.cu): components a selection may leave
@@ -92,6 +92,8 @@ struct SelCtl {
   uint32_t cmd, arrived;      // selections posted / passes finished (see minor_select.cu)
   uint32_t phases;            // passes of the tile so far in this run
   float near;                 // the tile's resolve margin
+  int32_t slow;               // selections running that the plain loop would have beaten
+  unsigned long long hand_key;  // the peak from which the plain loop takes the round on (0: none)
 };
 struct SelDev {
   float2* u;            // [T][cell_stride] bounds of R and -R per 8 x 8 cell
@@ -105,6 +107,8 @@ struct SelDev {
   int32_t lq, pitch;
   int32_t oy8, ox8, w8; // h8 and hb: entry of offset 0, row length
   int32_t inside;       // the PSF array holds every offset between two pixels of a tile
+  float plain_cycles;   // what the launch behind the selection needs for an iteration
+                        // (0: no such launch, the selection takes the whole round)
 };
 struct SelSizes {
   size_t cells, boxes, h8, hb, lobe, ctl;  // bytes
@@ -171,6 +175,8 @@ struct MinorCfg {
                       // in tensor memory for the launch (streamed pipeline)
   int32_t pair;       // 1: groups of 2G CTAs serve pairs of tiles, alternating
                       // between them (streamed pipeline, grid groups, T even)
+  int32_t takeover;   // 1: only tiles that the selection ahead handed over, from
+                      // there on (plain loads)
 };
 
 // Pipeline geometry and shared-memory size for a minor-loop configuration
@@ -208,6 +214,12 @@ cudaError_t launch_first_level(const PlanDev& d, cudaStream_t s);
 __host__ __device__ __forceinline__ bool feedback_on(const PlanDev& d) {
   return (d.K > 0 || d.trigger > 0.f) && d.T > 1;
 }
+// Rounds of several selections, which the plain loop may take over in groups that
+// hold their tile in shared memory (rounds that a flux trigger ends are short: an
+// idle launch each would cost 3 %).
+inline bool takeover_possible(const PlanDev& d) {
+  return d.T == 1 ? d.K == 0 || d.K > kSelPending : d.K > kSelPending && !(d.trigger > 0.f);
+}
 // r_map / p_map: 2-D tensor maps of the residual and the PSF with the box
 // (c.box_w x c.chunk_h) of a pipelined configuration (ignored otherwise).
 cudaError_t launch_minor(const PlanDev& d, const MinorCfg& c, int parity,
@@ -219,6 +231,9 @@ bool make_box_tensor_map(CUtensorMap* map, const float* base, int rows, int cols
 bool encode_tensor_map_2d(CUtensorMap* map, const float* base, int rows, int cols, int box_w,
                           int box_h);
 cudaError_t minor_prepare(const MinorCfg& c);  // sets function attributes
+// SM cycles of an iteration with plain loads and resident rows, for a tile of h x w
+// pixels on the group of c.
+float minor_plain_cycles(const MinorCfg& c, int h, int w);
 // ---- selection minor loop (minor_select.cu) -----------------------------------
 // Table geometry and buffer sizes for an image's tiling; false if a tile is
 // too large for the packed positions.
@@ -242,8 +257,10 @@ bool select_cluster_fits(int direct, int G, int smem);
 // per item), each reading its image's plan state from `plans` (device
 // arrays); resident: each CTA's rows fit `smem` bytes of shared memory.
 // Image i runs its round (round - plans[i].round0).
+// takeover: as in MinorCfg.
 cudaError_t launch_minor_batch(const PlanDev* plans, const BatchItem* items, int n_items,
-                               int G, int resident, int smem, int round, cudaStream_t s);
+                               int G, int resident, int smem, int takeover, int round,
+                               cudaStream_t s);
 // Largest cluster size <= want that can be scheduled for the batched kernel.
 int minor_batch_cluster(int want, int resident, int smem);
 

@@ -278,7 +278,14 @@ __device__ __forceinline__ void minor_body(const PlanDev& d, const MinorCfg& c, 
   if (*(volatile int32_t*)&d.st->status != 0) return;
 
   uint64_t key = d.peak[parity * d.T + t];
-  const int64_t budget = d.budget[t];
+  int64_t k0 = 0;  // the round's components so far
+  if (c.takeover) {
+    key = d.sel.ctl[t].hand_key;
+    if (key == 0ull) return;  // the same for the whole group
+    k0 = d.rcount[t];
+    if (rank == 0 && threadIdx.x == 0) atomicAdd(&d.st->taken_over, 1);
+  }
+  const int64_t budget = d.budget[t] + k0;  // at the round's start
   const int64_t kmax = (d.K > 0 && (int64_t)d.K < budget) ? (int64_t)d.K : budget;
   const float level = d.trigger > 0.f ? *(volatile float*)&d.st->level : 0.f;
   const uint32_t seq0 = d.gbar[t];  // the tile's exchanges so far in this run
@@ -297,7 +304,7 @@ __device__ __forceinline__ void minor_body(const PlanDev& d, const MinorCfg& c, 
   }
   __syncthreads();
 
-  int64_t k = 0;
+  int64_t k = k0;
   while (k < kmax && key != 0ull) {
     const float v = key_value(key);
     if (!(fabsf(v) > d.thr) || !(fabsf(v) > level)) break;  // threshold, flux trigger
@@ -320,7 +327,7 @@ __device__ __forceinline__ void minor_body(const PlanDev& d, const MinorCfg& c, 
     uint64_t mine = (best_a >= 0.f) ? make_key(best_v, best_i) : 0ull;
     mine = block_max_key(mine, s_warp);
 
-    key = exchange_keys<SYNC>(d, c, t, rank, k, seq0, mine, s_part, &s_best, &s_abort);
+    key = exchange_keys<SYNC>(d, c, t, rank, k - k0, seq0, mine, s_part, &s_best, &s_abort);
     if (s_abort) break;
     ++k;
   }
@@ -340,7 +347,7 @@ __device__ __forceinline__ void minor_body(const PlanDev& d, const MinorCfg& c, 
     d.rcount[t] = (int32_t)k;
     d.rapplied[t] = (int32_t)k;
     d.budget[t] = budget - k;
-    d.gbar[t] = seq0 + (uint32_t)k;
+    d.gbar[t] = seq0 + (uint32_t)(k - k0);
   }
 }
 
@@ -1663,9 +1670,11 @@ int minor_batch_cluster(int want, int resident, int smem) {
 }
 
 cudaError_t launch_minor_batch(const PlanDev* plans, const BatchItem* items, int n_items, int G,
-                               int resident, int smem, int round, cudaStream_t s) {
+                               int resident, int smem, int takeover, int round,
+                               cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
   MinorCfg c{};
+  c.takeover = takeover;
   c.G = G;
   c.sync = G > 1 ? CLEAN_SYNC_CLUSTER : kSyncNone;
   c.resident = resident;
@@ -1707,6 +1716,22 @@ cudaError_t minor_prepare(const MinorCfg& c) {
 }
 
 int minor_threads() { return kThreads; }
+
+// Fitted to the plain loop at 64^2 to 2048^2, groups of 1 to 152 CTAs (1.75 us
+// and 1.8 us a step of up to 8192 pixels, less where the threads of a row cover
+// more columns than the tile has; a grid exchange 0.9 us more than a cluster's,
+// and 10 ns a CTA from 32 on): within 10 % of the measured times, mostly below
+// them, so 8 % on top; 2 cycles a nanosecond.
+float minor_plain_cycles(const MinorCfg& c, int h, int w) {
+  int tpr = 32;
+  while (tpr < w && tpr < kThreads) tpr <<= 1;
+  const int rows = (h + c.G - 1) / c.G, per = kThreads / tpr * kUnroll;
+  const int cols = (w + tpr - 1) / tpr, steps = (rows + per - 1) / per * cols;
+  double us = 1.75 + 1.8 * steps * (0.45 + 0.55 * (double)w / ((double)tpr * cols));
+  if (steps == 1) us = std::min(us, 2.6 + (double)rows / per);
+  if (c.sync == CLEAN_SYNC_GRID) us += 0.9 + 0.01 * std::max(0, c.G - 32);
+  return (float)(us * 1.08 * 2000.0);
+}
 
 bool make_box_tensor_map(CUtensorMap* map, const float* base, int rows, int cols, int box_w,
                          int box_h) {

@@ -42,6 +42,15 @@
 // 4 x 4 cells), not of 4 x 4.  It does not fit shared memory and need not: its
 // L2 round trip runs beside the candidates'.
 //
+// Where the residual is flat, most cells come near the peak again and again, and
+// the resolves cost more than a pass over a small tile would (256^2 with 250
+// sources, 8000 iterations: 4.6 us an iteration against the plain loop's 3.1; with
+// 20 sources 2.5).  What decides is the run, not its parameters, so rank 0 times
+// its selections: after two running that cost more than the plain loop's
+// iterations (SelDev::plain_cycles) the tile's components are applied, the peak
+// is left in SelCtl::hand_key, and the launch behind this one goes on from there.
+// That field takes 3.05 us now, the sparse one 2.5.
+//
 // What bounds it: an iteration is a chain of about 1500 cycles (0.75 us: decode,
 // one L2 round trip of the candidates' PSF gather at one L1 tag a candidate,
 // two warp reductions either side of a barrier), 3400 with superblocks (the
@@ -85,6 +94,9 @@ constexpr int kManyCells = 32, kFewCells = 8;
 // a cell whose range depends on the peak's place within a cell: plus the cell's
 // place among the 8 x 8 around the peak (a NaN, so no pair that the table holds)
 constexpr uint32_t kLobeMark = 0xffc00000u;
+// a tile goes to the plain loop after this many selections running that cost
+// more than it would, if this many iterations of the round are left (see SelDev)
+constexpr int kSlowRuns = 2, kSlowLeft = 32;
 constexpr int kUnitRows = 8, kUnitCols = 32;  // pixels a warp takes at a time in a pass
 
 __device__ __forceinline__ uint32_t redux_max(uint32_t v) {
@@ -136,6 +148,7 @@ struct SelShared {
   unsigned long long key;     // the pass's peak key (this CTA's part)
   long long k_cmd;            // the group's command: components so far, finished
   int done_cmd, abort;
+  int slow;                   // selections running that the plain loop would have beaten
   // followed by the cells' PSF ranges (SelDev::h8) in tiles without superblocks
 };
 
@@ -1117,19 +1130,26 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
   const float level = d.trigger > 0.f ? *(volatile float*)&d.st->level : 0.f;
   SelCtl* ctl = d.sel.ctl + t;
   const uint32_t base = ctl->phases;
+  // tiles whose rounds the plain loop has taken over (the group reads this
+  // before rank 0 can change it: that is behind its wait for their passes)
+  const bool hand_all = d.sel.plain_cycles > 0.f && ctl->slow >= kSlowRuns;
   const bool idle = kmax <= 0 || key == 0ull || !(key_abs(key) > d.thr) || !(key_abs(key) > level);
   if (threadIdx.x == 0) {
     s.abort = 0;
     s.key = 0ull;
+    s.slow = ctl->slow;
   }
   for (int j = threadIdx.x; j < kPending + 16; j += kThreads) s.comp[j] = make_int4(0, 0, 0, 0);
   int64_t k = 0, applied = 0;  // components of the round; those the residual has
   uint32_t phase = 0;
-  bool done = idle;
+  bool done = idle, hand = false;
+  unsigned long long hand_key = key;
   __syncthreads();
-  while (!idle) {
+  if (hand_all) hand = !idle;
+  while (!idle && !hand) {
+    const long long t0 = clock64();
     // the pending components, then the cells (unless the round is over)
-    if (done && !flush) break;
+    if (done && (!flush || k == applied)) break;
     tile_pass(d, g, rank, G, (int)(k - applied), !done);
     applied = k;
     if (done) break;
@@ -1165,8 +1185,20 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
         abs0 = (uint32_t)(key >> 32);
         lo0 = cand_lo(((uint32_t)(py - g.rc.y0) << 15) | (uint32_t)(px - g.rc.x0), key_value(key));
       }
+      const bool over = s.slow >= kSlowRuns && kmax - k >= kSlowLeft;
       __syncthreads();
-      k += select_components<DIRECT>(d, g, t, abs0, lo0, k, kmax, level, &done);
+      if (over) {
+        // nothing is pending: the plain loop goes on from this peak
+        const uint32_t p = lo_pos(lo0);
+        hand_key = make_key(__uint_as_float(abs0 | (lo0 << 31)),
+                            (g.rc.y0 + (int)(p >> 15)) * d.nx + g.rc.x0 + (int)(p & 0x7fffu));
+        hand = done = true;
+      } else {
+        const int n = select_components<DIRECT>(d, g, t, abs0, lo0, k, kmax, level, &done);
+        k += n;
+        if (threadIdx.x == 0 && d.sel.plain_cycles > 0.f && !done)
+          s.slow = (float)(clock64() - t0) > d.sel.plain_cycles * (float)n ? s.slow + 1 : 0;
+      }
       if (threadIdx.x == 0) {
         s.key = 0ull;
         if (G > 1) {
@@ -1208,6 +1240,8 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
     d.rapplied[t] = (int32_t)applied;
     d.budget[t] = budget - k;
     ctl->phases = base + phase;
+    ctl->slow = s.slow;
+    ctl->hand_key = hand && !s.abort ? hand_key : 0ull;
   }
 }
 

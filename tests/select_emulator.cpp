@@ -190,6 +190,7 @@ static void atomicMax(unsigned long long* p, unsigned long long v) {
 }
 static void __threadfence() {}
 static void __nanosleep(unsigned) { sched_yield(); }
+static long long clock64() { return std::chrono::steady_clock::now().time_since_epoch().count(); }
 using std::max;
 using std::min;
 
@@ -229,13 +230,14 @@ static void launch(int blocks, int threads, size_t smem, const std::function<voi
 }
 
 int main(int argc, char** argv) {
-  // ny nx psf_ny psf_nx tiles_y tiles_x G, niter, gain threshold; dirty; PSF
+  // ny nx psf_ny psf_nx tiles_y tiles_x G, niter, gain threshold plain_cycles;
+  // dirty; PSF
   std::FILE* f = std::fopen(argv[1], "rb");
   int32_t n[7];
   int64_t niter;
-  float gt[2];
+  float gt[3];
   if (argc < 3 || !f || std::fread(n, 4, 7, f) != 7 || std::fread(&niter, 8, 1, f) != 1 ||
-      std::fread(gt, 4, 2, f) != 2)
+      std::fread(gt, 4, 3, f) != 3)
     return 2;
   PlanDev d{};
   d.ny = n[0], d.nx = n[1], d.pny = n[2], d.pnx = n[3], d.ty = n[4], d.tx = n[5];
@@ -278,6 +280,7 @@ int main(int argc, char** argv) {
   d.rcomps = rcomps.data(), d.st = &st;
   d.sel.u = (float2*)u.data(), d.sel.masks = (uint2*)masks.data(), d.sel.ctl = (SelCtl*)ctl.data();
   d.sel.h8 = (uint32_t*)h8.data(), d.sel.hb = (uint32_t*)hb.data(), d.sel.lobe = (uint32_t*)lobe.data();
+  d.sel.plain_cycles = gt[2];
   d.sel.inside = d.cy >= maxH - 1 && d.pny - d.cy >= maxH && d.cx >= maxW - 1 && d.pnx - d.cx >= maxW;
 
   // the PSF's tables (select_build_psf)
@@ -321,6 +324,7 @@ int main(int argc, char** argv) {
   std::fwrite(model.data(), 4, model.size(), f);
   for (int t = 0; t < d.T; ++t) {
     std::fwrite(&rcount[t], 4, 1, f);
+    std::fwrite(&d.sel.ctl[t].hand_key, 8, 1, f);
     std::fwrite(&rcomps[(size_t)t * d.cap_round], sizeof(clean_component), rcount[t], f);
   }
   std::fclose(f);

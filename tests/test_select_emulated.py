@@ -65,11 +65,12 @@ def emulator(tmp_path_factory):
     return build
 
 
-def _emulate(exe, tmp_path, dirty, psf, gain, niter, thr, tiles, G):
+def _emulate(exe, tmp_path, dirty, psf, gain, niter, thr, tiles, G, plain_cycles=0.0):
+    """(residual, model, components, tiles' hand-over keys) of one launch."""
     ny, nx = dirty.shape
     inp, out = tmp_path / "in", tmp_path / "out"
     inp.write_bytes(np.array([ny, nx, *psf.shape, *tiles, G], np.int32).tobytes()
-                    + np.int64(niter).tobytes() + np.array([gain, thr], np.float32).tobytes()
+                    + np.int64(niter).tobytes() + np.array([gain, thr, plain_cycles], np.float32).tobytes()
                     + dirty.tobytes() + psf.tobytes())
     r = subprocess.run([exe, str(inp), str(out)], capture_output=True, text=True, timeout=600,
                        env=dict(os.environ, TSAN_OPTIONS="halt_on_error=0 exitcode=66"))
@@ -79,12 +80,13 @@ def _emulate(exe, tmp_path, dirty, psf, gain, niter, thr, tiles, G):
     b = out.read_bytes()
     n = ny * nx
     f = np.frombuffer(b, np.float32, 2 * n)
-    comps, at = [], 8 * n
+    comps, keys, at = [], [], 8 * n
     for _ in range(tiles[0] * tiles[1]):
         k = int(np.frombuffer(b, np.int32, 1, at)[0])
-        comps.append(np.frombuffer(b, cg.COMPONENT_DTYPE, k, at + 4))
-        at += 4 + 16 * k
-    return f[:n].reshape(ny, nx), f[n:].reshape(ny, nx), np.concatenate(comps)
+        keys.append(int(np.frombuffer(b, np.uint64, 1, at + 4)[0]))
+        comps.append(np.frombuffer(b, cg.COMPONENT_DTYPE, k, at + 12))
+        at += 12 + 16 * k
+    return f[:n].reshape(ny, nx), f[n:].reshape(ny, nx), np.concatenate(comps), keys
 
 
 def _field(ny, nx, ps, seed):
@@ -103,7 +105,8 @@ def _field(ny, nx, ps, seed):
 def _check(emulator, tmp_path, dirty, psf, niter, thr=0.0, tiles=(1, 1), G=1, threads=64,
            gain=0.1):
     o = oracle.clean_f32(dirty, psf, gain, niter, thr, tiles, 0)
-    r, m, c = _emulate(emulator(threads), tmp_path, dirty, psf, gain, niter, thr, tiles, G)
+    r, m, c, keys = _emulate(emulator(threads), tmp_path, dirty, psf, gain, niter, thr, tiles, G)
+    assert not any(keys)
     for k in ("y", "x", "tile"):
         assert np.array_equal(c[k], o.comps[k]), (k, c[k], o.comps[k])
     assert np.array_equal(c["flux"].view(np.uint32), o.comps["flux"].view(np.uint32))
@@ -152,3 +155,20 @@ def test_cells_with_nan_pixels(emulator, tmp_path):
     psf = np.zeros((3, 3), np.float32)
     psf[1, 1] = psf[1, 2] = 400.0
     _check(emulator, tmp_path, dirty, psf, 12)
+
+
+@pytest.mark.parametrize("G", [1, 2])
+def test_tile_handed_over_to_the_plain_loop(emulator, tmp_path, G):
+    """Against a plain loop that costs nothing every selection is slow: after
+    two the round stops, the residual holds every component, and the key is
+    that of its peak."""
+    dirty, psf = _field(48, 40, (96, 80), 3)
+    r, m, c, (key,) = _emulate(emulator(64), tmp_path, dirty, psf, 0.1, 300, 0.0, (1, 1), G, 1e-6)
+    assert 2 <= len(c) <= 128
+    o = oracle.clean_f32(dirty, psf, 0.1, len(c), 0.0, (1, 1), 0)
+    assert np.array_equal(c["y"], o.comps["y"]) and np.array_equal(c["x"], o.comps["x"])
+    assert np.array_equal(r.view(np.uint32), o.residual.view(np.uint32))
+    assert np.array_equal(m.view(np.uint32), o.model.view(np.uint32))
+    i = int(np.abs(r).argmax())
+    v = int(r.ravel()[i].view(np.uint32))
+    assert key == ((v & 0x7fffffff) << 32 | (0x7fffffff - i) << 1 | v >> 31)
