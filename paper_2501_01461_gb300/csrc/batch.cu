@@ -63,12 +63,17 @@ struct Group {
 // Shared engine behind both APIs.
 struct clean_engine_s {
   int device = 0;
+  int sms = 0;
+  int room[5] = {0, 0, 0, 0, 0};  // clusters of 1 << i CTAs that run at once, one CTA
+                                  // an SM (room[1] 0: not asked yet)
   int cap = 0;                          // state slots
   std::vector<Job> jobs;                // resident jobs (finished ones until removed)
   std::vector<int> free_slots;
   DevState* d_states = nullptr;         // [cap] control blocks
   DevState* h_states = nullptr;         // pinned mirror
   bool states_read = false;             // it is as the device's: nothing launched since
+  int32_t* d_handed = nullptr;          // tiles handed over in a round (SelDev::handed)
+  bool takeovers = false;               // a launch takes tiles over
   PlanDev* d_plans = nullptr;           // [cap] device copies, indexed by work position
   BatchItem* d_items = nullptr;
   int items_cap = 0;
@@ -115,6 +120,7 @@ void engine_free(clean_engine_s* e) {
   if (e->cap_stream) cudaStreamDestroy(e->cap_stream);
   for (Job& j : e->jobs) clean_destroy(j.plan);
   cudaFree(e->d_states);
+  cudaFree(e->d_handed);
   cudaFree(e->d_plans);
   cudaFree(e->d_items);
   cudaFree(e->d_imgs);
@@ -129,8 +135,10 @@ int engine_create(clean_engine_s** out, int cap) {
   if (!e) return CLEAN_ERR_OOM;
   e->cap = cap;
   cudaGetDevice(&e->device);
+  cudaDeviceGetAttribute(&e->sms, cudaDevAttrMultiProcessorCount, e->device);
   if (cudaMalloc(&e->d_states, sizeof(DevState) * cap) != cudaSuccess ||
       cudaMallocHost(&e->h_states, sizeof(DevState) * cap) != cudaSuccess ||
+      cudaMalloc(&e->d_handed, sizeof(int32_t)) != cudaSuccess ||
       cudaMalloc(&e->d_plans, sizeof(PlanDev) * cap) != cudaSuccess ||
       cudaMalloc(&e->d_imgs, sizeof(BatchImage) * cap) != cudaSuccess ||
       cudaMalloc(&e->d_maps, sizeof(CUtensorMap) * cap) != cudaSuccess) {
@@ -205,6 +213,16 @@ void tile_group(int h, int w, int* G, int* resident, int* smem) {
   *smem = 0;
 }
 
+// CTAs (a power of two up to 16) that n tiles may have in clusters and still run at
+// once.  Clusters need their SMs together: there is room for 7 of 16, 15 of 8, 36 of 4.
+int cluster_room(clean_engine_s* e, int64_t n) {
+  if (e->room[1] == 0)
+    for (int i = 1; i < 5; ++i) e->room[i] = minor_batch_clusters(1 << i, 1, (int)kGroupSmemMax);
+  int i = 0;
+  while (i < 4 && e->room[i + 1] >= n) ++i;
+  return 1 << i;
+}
+
 // The same for a launch that takes tiles over from their selections: where SMs
 // are idle (`most` a tile), more CTAs, down to 2048 pixels each.
 void takeover_group(int h, int w, int most, int* G, int* resident, int* smem) {
@@ -215,15 +233,15 @@ void takeover_group(int h, int w, int most, int* G, int* resident, int* smem) {
   }
 }
 
-// CTAs per tile of a selection.  With at most kSelPending iterations a round
-// the tile is scanned once and the rest is one CTA's; a round of several
-// selections passes over the tile between them, which a cluster shares (about
-// 4096 pixels a CTA; at most 8, the portable cluster size).
-int select_group(const PlanDev& d) {
-  if (d.K > 0 && d.K <= kSelPending) return 1;
+// CTAs per tile of a selection, as far as SMs are idle (`most` a tile).  They share
+// the passes over the tile: one a round with at most kSelPending iterations (16384
+// pixels a CTA), one between any two selections of longer rounds (4096).  A power
+// of two: images of about a size share a launch.
+int select_group(const PlanDev& d, int64_t most) {
   const Rect r = tile_rect(0, d.ny, d.nx, d.ty, d.tx);
+  const int64_t per = d.K > 0 && d.K <= kSelPending ? 16384 : 4096;
   int G = 1;
-  while (G < 8 && (int64_t)G * 4096 < (int64_t)(r.y1 - r.y0) * (r.x1 - r.x0)) G *= 2;
+  while (2 * G <= most && G * per < (int64_t)(r.y1 - r.y0) * (r.x1 - r.x0)) G *= 2;
   return G;
 }
 
@@ -254,14 +272,17 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
   std::vector<Sized> all;
   int block0 = 0;
   e->blocks_tma = e->blocks_plain = 0;
-  int sms = 0;
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, e->device);
-  int64_t n_tiles = 0;
-  for (int w : work) n_tiles += e->jobs[w].dev.T;
+  int64_t n_tiles = 0, n_over = 0;
+  for (int w : work) {
+    n_tiles += e->jobs[w].dev.T;
+    if (takeover_possible(e->jobs[w].dev)) n_over += e->jobs[w].dev.T;
+  }
+  const int most_over = n_over ? cluster_room(e, n_over) : 1;
   for (int w = 0; w < (int)work.size(); ++w) {
     Job& j = e->jobs[work[w]];
     plans.push_back(j.dev);
-    plans.back().sel.plain_cycles = 0.f;  // (its own launches' value)
+    plans.back().sel.plain_cycles = 0.f;  // (its own launches' values)
+    plans.back().sel.handed = nullptr;
     maps.push_back(j.map);
     if (j.fft)
       e->fft_work.push_back(w);
@@ -269,19 +290,20 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
       ++e->n_gather;
     if (j.tma && !j.fft) ++e->n_tma;
     e->max_T = std::max(e->max_T, j.dev.T);
-    const int sel_G = j.sel_smem ? select_group(j.dev) : 0;
+    const int sel_G = j.sel_smem ? select_group(j.dev, e->sms / n_tiles) : 0;
     // behind the selections: the plain loop, for tiles on which it is the faster
     // (see minor_select.cu); one group size for the image
     Sized takeover{};
     if (j.sel_smem && takeover_possible(j.dev)) {
       const int h = (j.dev.ny + j.dev.ty - 1) / j.dev.ty, wd = (j.dev.nx + j.dev.tx - 1) / j.dev.tx;
       takeover.takeover = 1;
-      takeover_group(h, wd, (int)(sms / n_tiles), &takeover.G, &takeover.resident, &takeover.smem);
+      takeover_group(h, wd, most_over, &takeover.G, &takeover.resident, &takeover.smem);
       if (takeover.resident) {
         MinorCfg c{};
         c.G = takeover.G;
         c.sync = CLEAN_SYNC_CLUSTER;
         plans.back().sel.plain_cycles = minor_plain_cycles(c, h, wd);
+        plans.back().sel.handed = e->d_handed;
       }
     }
     for (int t = 0; t < j.dev.T; ++t) {
@@ -321,7 +343,7 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
   }
   // groups of one launch each, biggest tiles first within each
   auto kind = [](const Sized& z) {
-    return (((1 - z.takeover) * 2 + z.select) * 2 + z.direct) * 64 + z.resident * 32 + z.G;
+    return ((((1 - z.takeover) * 2 + z.select) * 2 + z.direct) * 2 + z.resident) * 1024 + z.G;
   };
   std::stable_sort(all.begin(), all.end(), [&](const Sized& a, const Sized& b) {
     return kind(a) != kind(b) ? kind(a) > kind(b) : a.px > b.px;
@@ -344,16 +366,18 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
     ++g.count;
     items.push_back(all[k].it);
   }
+  e->takeovers = false;
   for (size_t k = e->groups.size(); k-- > 0;) {
-    // a cluster size the device cannot schedule
     const Group& g = e->groups[k];
-    if (g.G == 1 || (g.select ? select_cluster_fits(g.direct, g.G, g.smem)
-                              : minor_batch_cluster(g.G, g.resident, g.smem) == g.G))
+    if (!g.select && g.G > 1 && minor_batch_clusters(g.G, g.resident, g.smem) < 1) {
+      // a cluster size the device cannot schedule
+      if (!g.takeover) return CLEAN_ERR_UNSUPPORTED;
+      for (int i = g.offset; i < g.offset + g.count; ++i)  // selections take the whole rounds
+        plans[items[i].image].sel.plain_cycles = 0.f;
+      e->groups.erase(e->groups.begin() + (long)k);
       continue;
-    if (!g.takeover) return CLEAN_ERR_UNSUPPORTED;
-    for (int i = g.offset; i < g.offset + g.count; ++i)  // the selections take the whole rounds
-      plans[items[i].image].sel.plain_cycles = 0.f;
-    e->groups.erase(e->groups.begin() + (long)k);
+    }
+    e->takeovers |= g.takeover != 0;
   }
   if ((int)items.size() > e->items_cap) {
     cudaFree(e->d_items);
@@ -425,7 +449,8 @@ int engine_mark(clean_engine_s* e) {
 // Launches `rounds` rounds of every unfinished job.
 // The kernels of one round (round index `round`) on stream s; *n counts them.
 cudaError_t launch_round(clean_engine_s* e, int round, cudaStream_t s, int* n) {
-  cudaError_t err = cudaSuccess;
+  cudaError_t err = e->takeovers ? cudaMemsetAsync(e->d_handed, 0, sizeof(int32_t), s) : cudaSuccess;
+  if (err != cudaSuccess) return err;
   for (const Group& g : e->groups) {
     err = g.select ? launch_select_batch(e->d_plans, e->d_items + g.offset, g.count, g.direct, g.G,
                                          g.smem, round, 2000000000ull, s)

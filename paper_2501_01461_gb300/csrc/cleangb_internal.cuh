@@ -89,7 +89,8 @@ struct SelCtl {
   unsigned long long key[2];  // peak key of a pass, by the pass's parity
   int64_t k;                  // the posted selection: components of the round so far
   int32_t done;               // the round is over for the tile
-  uint32_t cmd, arrived;      // selections posted / passes finished (see minor_select.cu)
+  uint32_t cmd, arrived;      // selections posted, CTAs that finished a pass (see
+                              // minor_select.cu)
   uint32_t phases;            // passes of the tile so far in this run
   float near;                 // the tile's resolve margin
   int32_t slow;               // selections running that the plain loop would have beaten
@@ -107,6 +108,7 @@ struct SelDev {
   int32_t lq, pitch;
   int32_t oy8, ox8, w8; // h8 and hb: entry of offset 0, row length
   int32_t inside;       // the PSF array holds every offset between two pixels of a tile
+  int32_t* handed;      // tiles handed over in the launch (batches; null: not counted)
   float plain_cycles;   // what the launch behind the selection needs for an iteration
                         // (0: no such launch, the selection takes the whole round)
 };
@@ -246,12 +248,11 @@ cudaError_t select_prepare();  // kernel attributes
 // leave no component pending.
 cudaError_t launch_select(const PlanDev& d, int G, int smem, int parity, int flush, uint64_t limit_ns,
                           int force_timeout, cudaStream_t s);
-// G CTAs per (image, tile) item (G > 1: one cluster each); direct: tiles without
-// superblocks (SelDev::lq 0).
+// G CTAs per (image, tile) item (G > 1: a cooperative launch, every CTA on an SM of
+// its own); direct: tiles without superblocks (SelDev::lq 0).
 cudaError_t launch_select_batch(const PlanDev* plans, const BatchItem* items, int n_items,
                                 int direct, int G, int smem, int round, uint64_t limit_ns,
                                 cudaStream_t s);
-bool select_cluster_fits(int direct, int G, int smem);
 
 // G CTAs per item (G = 1: independent CTAs; G > 1: one thread-block cluster
 // per item), each reading its image's plan state from `plans` (device
@@ -261,8 +262,8 @@ bool select_cluster_fits(int direct, int G, int smem);
 cudaError_t launch_minor_batch(const PlanDev* plans, const BatchItem* items, int n_items,
                                int G, int resident, int smem, int takeover, int round,
                                cudaStream_t s);
-// Largest cluster size <= want that can be scheduled for the batched kernel.
-int minor_batch_cluster(int want, int resident, int smem);
+// Clusters of G CTAs of the batched kernel that the device runs at once.
+int minor_batch_clusters(int G, int resident, int smem);
 
 // Feedback for many images in one launch (plain loads, or TMA when maps is
 // non-NULL: one PSF tensor map per image in device memory, 64-byte aligned).

@@ -1644,29 +1644,27 @@ const void* batch_fn(int G, int resident) {
 }
 }  // namespace
 
-int minor_batch_cluster(int want, int resident, int smem) {
-  for (int G = std::min(16, std::max(1, want)); G > 1; G /= 2) {
-    const void* fn = batch_fn(G, resident);
-    if (allow_max_smem(fn) != cudaSuccess) break;
-    if (G > 8 && cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-                     cudaSuccess)
-      continue;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(G, 1, 1);
-    cfg.blockDim = dim3(kThreads, 1, 1);
-    cfg.dynamicSmemBytes = resident ? smem : 0;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = G;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess && n >= 1) return G;
-  }
+int minor_batch_clusters(int G, int resident, int smem) {
+  const void* fn = batch_fn(G, resident);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(G, 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = resident ? smem : 0;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = G;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (allow_max_smem(fn) == cudaSuccess &&
+      (G <= 8 || cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+                     cudaSuccess) &&
+      cudaOccupancyMaxActiveClusters(&n, fn, &cfg) == cudaSuccess)
+    return n;
   cudaGetLastError();
-  return 1;
+  return 0;
 }
 
 cudaError_t launch_minor_batch(const PlanDev* plans, const BatchItem* items, int n_items, int G,

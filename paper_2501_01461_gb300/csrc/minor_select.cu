@@ -97,6 +97,7 @@ constexpr uint32_t kLobeMark = 0xffc00000u;
 // a tile goes to the plain loop after this many selections running that cost
 // more than it would, if this many iterations of the round are left (see SelDev)
 constexpr int kSlowRuns = 2, kSlowLeft = 32;
+constexpr float kFollow = 0.75f;
 constexpr int kUnitRows = 8, kUnitCols = 32;  // pixels a warp takes at a time in a pass
 
 __device__ __forceinline__ uint32_t redux_max(uint32_t v) {
@@ -148,6 +149,7 @@ struct SelShared {
   unsigned long long key;     // the pass's peak key (this CTA's part)
   long long k_cmd;            // the group's command: components so far, finished
   int done_cmd, abort;
+  long long t0;               // when the pass began
   int slow;                   // selections running that the plain loop would have beaten
   // followed by the cells' PSF ranges (SelDev::h8) in tiles without superblocks
 };
@@ -1091,9 +1093,10 @@ __device__ __forceinline__ int select_components(const PlanDev& d, const Geo& g,
 // The tile's CTAs share its passes; rank 0 selects.  After each pass every
 // other rank counts itself in (SelCtl::arrived) and rank 0 waits for the
 // count; after each selection rank 0 posts the component count and whether
-// the round is over (SelCtl::cmd) and the others wait for the post.  Both
-// count on across launches (base: passes of the tile so far).  Waits are
-// bounded by limit_ns; an expired one sets ST_TIMEOUT.
+// the round is over (SelCtl::cmd) and the others wait for the post.  The posts
+// count on across launches (base: passes of the tile so far), the arrivals start
+// again in each, so that a tile's group may have another size in the next round.
+// Waits are bounded by limit_ns; an expired one sets ST_TIMEOUT.
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
   uint32_t v;
@@ -1113,6 +1116,14 @@ __device__ __forceinline__ bool wait_count(const uint32_t* p, uint32_t want, uin
     if (ld_acquire(p) == want) return true;
     if (ptx::globaltimer_ns() - t0 > limit_ns) return false;
   }
+}
+
+// The cycles a component above which the plain loop is preferred.  In a batch its
+// launch waits for the last image's selections, so once one has gone over the
+// others follow unless they are a good deal faster.
+__device__ __forceinline__ float slow_above(const PlanDev& d) {
+  const bool follow = d.sel.handed && *(volatile int32_t*)d.sel.handed > 0;
+  return follow ? kFollow * d.sel.plain_cycles : d.sel.plain_cycles;
 }
 
 // CTA `rank` of the G serving tile t for one round.  flush: leave no
@@ -1138,16 +1149,15 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
     s.abort = 0;
     s.key = 0ull;
     s.slow = ctl->slow;
+    if (rank == 0) ctl->hand_key = hand_all && !idle ? key : 0ull;
   }
   for (int j = threadIdx.x; j < kPending + 16; j += kThreads) s.comp[j] = make_int4(0, 0, 0, 0);
   int64_t k = 0, applied = 0;  // components of the round; those the residual has
   uint32_t phase = 0;
-  bool done = idle, hand = false;
-  unsigned long long hand_key = key;
+  bool done = idle;
   __syncthreads();
-  if (hand_all) hand = !idle;
-  while (!idle && !hand) {
-    const long long t0 = clock64();
+  while (!idle && !hand_all) {
+    if (threadIdx.x == 0) s.t0 = clock64();
     // the pending components, then the cells (unless the round is over)
     if (done && (!flush || k == applied)) break;
     tile_pass(d, g, rank, G, (int)(k - applied), !done);
@@ -1163,8 +1173,7 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
         atomicAdd(&ctl->arrived, 1u);
       } else {
         if (!wait_count(&ctl->arrived,
-                        (base + phase) * (uint32_t)(G - 1) + (force_timeout ? 1u : 0u), limit_ns,
-                        false)) {
+                        phase * (uint32_t)(G - 1) + (force_timeout ? 1u : 0u), limit_ns, false)) {
           atomicOr(&d.st->status, ST_TIMEOUT);
           d.st->timeout_where = ((int64_t)t << 32) | (int64_t)k;
           s.abort = 1;
@@ -1190,14 +1199,17 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
       if (over) {
         // nothing is pending: the plain loop goes on from this peak
         const uint32_t p = lo_pos(lo0);
-        hand_key = make_key(__uint_as_float(abs0 | (lo0 << 31)),
-                            (g.rc.y0 + (int)(p >> 15)) * d.nx + g.rc.x0 + (int)(p & 0x7fffu));
-        hand = done = true;
+        if (threadIdx.x == 0) {
+          ctl->hand_key = make_key(__uint_as_float(abs0 | (lo0 << 31)),
+                                   (g.rc.y0 + (int)(p >> 15)) * d.nx + g.rc.x0 + (int)(p & 0x7fffu));
+          if (d.sel.handed) atomicAdd(d.sel.handed, 1);
+        }
+        done = true;
       } else {
         const int n = select_components<DIRECT>(d, g, t, abs0, lo0, k, kmax, level, &done);
         k += n;
         if (threadIdx.x == 0 && d.sel.plain_cycles > 0.f && !done)
-          s.slow = (float)(clock64() - t0) > d.sel.plain_cycles * (float)n ? s.slow + 1 : 0;
+          s.slow = (float)(clock64() - s.t0) > slow_above(d) * (float)n ? s.slow + 1 : 0;
       }
       if (threadIdx.x == 0) {
         s.key = 0ull;
@@ -1240,8 +1252,9 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
     d.rapplied[t] = (int32_t)applied;
     d.budget[t] = budget - k;
     ctl->phases = base + phase;
+    ctl->arrived = 0u;  // (every wait for it is over)
     ctl->slow = s.slow;
-    ctl->hand_key = hand && !s.abort ? hand_key : 0ull;
+    if (s.abort) ctl->hand_key = 0ull;
   }
 }
 
@@ -1252,7 +1265,7 @@ __global__ void __launch_bounds__(kThreads, 1)
                       (int)blockIdx.x % G);
 }
 
-// G CTAs per (image, tile) item; with G > 1 they form one cluster, so they run
+// G CTAs per (image, tile) item; with G > 1 the launch is cooperative, so they run
 // at the same time and may wait for each other.
 template <bool DIRECT>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -1449,47 +1462,25 @@ cudaError_t launch_select(const PlanDev& d, int G, int smem, int parity, int flu
       args);
 }
 
-namespace {
-void batch_config(cudaLaunchConfig_t* cfg, cudaLaunchAttribute* at, int n_items, int G, int smem) {
-  *cfg = cudaLaunchConfig_t{};
-  cfg->gridDim = dim3((unsigned)(n_items * G), 1, 1);
-  cfg->blockDim = dim3(kThreads, 1, 1);
-  cfg->dynamicSmemBytes = smem;
-  at->id = cudaLaunchAttributeClusterDimension;
-  at->val.clusterDim.x = G;
-  at->val.clusterDim.y = 1;
-  at->val.clusterDim.z = 1;
-  cfg->attrs = at;
-  cfg->numAttrs = G > 1 ? 1 : 0;
-}
-const void* batch_fn(int direct) {
-  return direct ? (const void*)select_batch_kernel<true> : (const void*)select_batch_kernel<false>;
-}
-}  // namespace
-
-bool select_cluster_fits(int direct, int G, int smem) {
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute at;
-  batch_config(&cfg, &at, 1, G, smem);
-  int n = 0;
-  if (cudaOccupancyMaxActiveClusters(&n, batch_fn(direct), &cfg) != cudaSuccess) {
-    cudaGetLastError();
-    return false;
-  }
-  return n >= 1;
-}
-
 cudaError_t launch_select_batch(const PlanDev* plans, const BatchItem* items, int n_items,
                                 int direct, int G, int smem, int round, uint64_t limit_ns,
                                 cudaStream_t s) {
   if (n_items <= 0) return cudaSuccess;
-  cudaLaunchConfig_t cfg;
-  cudaLaunchAttribute at;
-  batch_config(&cfg, &at, n_items, G, smem);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(n_items * G), 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = G > 1 ? 1 : 0;
   void* args[] = {const_cast<PlanDev**>(&plans), const_cast<BatchItem**>(&items), &G, &round,
                   &limit_ns};
-  return cudaLaunchKernelExC(&cfg, batch_fn(direct), args);
+  return cudaLaunchKernelExC(&cfg, direct ? (const void*)select_batch_kernel<true>
+                                          : (const void*)select_batch_kernel<false>,
+                             args);
 }
 
 }  // namespace cleangb
