@@ -428,7 +428,8 @@ CLEAN_API const char* clean_strerror(int status);
  *                              Same results, bit for bit.
  *   CLEAN_DEBUG_MINOR_PATH     minor-loop kernel: 0 automatic (selection when
  *                              group_ctas and group_sync are left to the
- *                              library and no tile side is above 32767; else
+ *                              library, no tile side is above 32767 and a
+ *                              round has more than a few iterations; else
  *                              the bulk-copy pipeline when image and PSF rows
  *                              are 16-byte aligned), 1 plain loads, 2 pipeline
  *                              when possible (same results, bit for bit)

@@ -49,6 +49,7 @@ struct clean_plan_s {
   // selection minor loop (minor_select.cu): the automatic choice whenever the
   // caller leaves the group to the library
   bool sel_ok = false;
+  bool sel_short = false;      // rounds too short for it (short_rounds)
   int sel_G = 1;               // CTAs per tile
   int sel_smem = 0;
   float2* sel_boxes = nullptr; // work area of the PSF tables
@@ -313,10 +314,28 @@ bool use_pipe(const clean_plan_s* pl) {
   return !pl->mc_pipe.resident;
 }
 
+// Whether rounds are too short to pay for a selection.  Its start (the tile's
+// cells scanned, the first candidates) costs about 14 us more than the plain
+// loop's, and 1 us more per 152,000 pixels of a tile; an iteration then saves all
+// but about 1 us of the plain loop's.  Measured, selection against plain loop, a
+// tile's iteration with K 4 and K 8: 150^2 tiles 9.7 / 8.2 and 6.0 / 6.3 us,
+// 512^2 untiled 9.8 / 9.3 and 6.0 / 7.6, 2048^2 untiled 21.0 / 19.9 and 14.0 / 17.9.
+// One iteration needs no candidates: equal at 512^2, 33.5 / 41.3 at 2048^2.
+// Streamed tiles (the pipeline): 90.4 / 89.7 with K 4 at 1024^2, 84.0 / 84.6 with 5.
+bool short_rounds(const clean_plan_s* pl) {
+  const int K = pl->d.K;
+  if (K == 0) return false;
+  if (!pl->mc.resident) return K <= 4;
+  const int h = max_extent(pl->p.ny, pl->p.tiles_y), w = max_extent(pl->p.nx, pl->p.tiles_x);
+  const double px = (double)h * w, plain_us = minor_plain_cycles(pl->mc, h, w) * 0.0005;
+  if (K == 1) return px <= 262144.0;
+  return K < 1.1 * (14.0 + px / 152000.0) / (plain_us - 1.0);
+}
+
 // Selection whenever the caller left the tile groups and the minor-loop
-// variant to the library.
+// variant to the library, and rounds are long enough.
 bool use_select(const clean_plan_s* pl) {
-  return pl->sel_ok && pl->minor_path == 0 && pl->p.group_ctas == 0 &&
+  return pl->sel_ok && !pl->sel_short && pl->minor_path == 0 && pl->p.group_ctas == 0 &&
          pl->p.group_sync == CLEAN_SYNC_AUTO;
 }
 
@@ -912,6 +931,7 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
   d.sel.lobe = pl->sel_lobe;
   d.sel.inside = d.cy >= maxH - 1 && d.pny - d.cy >= maxH && d.cx >= maxW - 1 &&
                  d.pnx - d.cx >= maxW;
+  pl->sel_short = short_rounds(pl);
   if (mc.resident && takeover_possible(d)) d.sel.plain_cycles = minor_plain_cycles(mc, maxH, maxW);
 
   if (pl->fft && (fft_make_twiddles(pl->fft_twy, pl->fft_ay, s) != cudaSuccess ||
