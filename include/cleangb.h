@@ -455,9 +455,10 @@ CLEAN_API const char* clean_strerror(int status);
  *                              taken to cost (a tile whose selections cost more
  *                              is handed over to it; 0: none is);
  *                              CLEAN_ERR_INVALID_ARG where the plan has no such
- *                              launch (several tiles with rounds of up to 64
- *                              iterations or a flux trigger, or tiles too large
- *                              for its groups' shared memory).  Same results,
+ *                              launch (fewer than 256 iterations a tile, several
+ *                              tiles with rounds of up to 64 iterations or a
+ *                              flux trigger, or tiles too large for its groups'
+ *                              shared memory).  Same results,
  *                              bit for bit.
  *   CLEAN_DEBUG_TIMING         1: bracket every minor-loop and feedback launch
  *                              with CUDA events on its stream and sum their

@@ -275,7 +275,7 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
   int64_t n_tiles = 0, n_over = 0;
   for (int w : work) {
     n_tiles += e->jobs[w].dev.T;
-    if (takeover_possible(e->jobs[w].dev)) n_over += e->jobs[w].dev.T;
+    if (takeover_possible(e->jobs[w].dev, plan_niter(e->jobs[w].plan))) n_over += e->jobs[w].dev.T;
   }
   const int most_over = n_over ? cluster_room(e, n_over) : 1;
   for (int w = 0; w < (int)work.size(); ++w) {
@@ -294,7 +294,7 @@ int engine_rebuild(clean_engine_s* e, cudaStream_t s) {
     // behind the selections: the plain loop, for tiles on which it is the faster
     // (see minor_select.cu); one group size for the image
     Sized takeover{};
-    if (j.sel_smem && takeover_possible(j.dev)) {
+    if (j.sel_smem && takeover_possible(j.dev, plan_niter(j.plan))) {
       const int h = (j.dev.ny + j.dev.ty - 1) / j.dev.ty, wd = (j.dev.nx + j.dev.tx - 1) / j.dev.tx;
       takeover.takeover = 1;
       takeover_group(h, wd, most_over, &takeover.G, &takeover.resident, &takeover.smem);

@@ -932,7 +932,7 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
   d.sel.inside = d.cy >= maxH - 1 && d.pny - d.cy >= maxH && d.cx >= maxW - 1 &&
                  d.pnx - d.cx >= maxW;
   pl->sel_short = short_rounds(pl);
-  if (mc.resident && takeover_possible(d)) d.sel.plain_cycles = minor_plain_cycles(mc, maxH, maxW);
+  if (mc.resident && takeover_possible(d, p->niter)) d.sel.plain_cycles = minor_plain_cycles(mc, maxH, maxW);
 
   if (pl->fft && (fft_make_twiddles(pl->fft_twy, pl->fft_ay, s) != cudaSuccess ||
                   fft_make_twiddles(pl->fft_twx, pl->fft_ax, s) != cudaSuccess)) {
@@ -1393,7 +1393,7 @@ int clean_debug_set(clean_plan_t pl, int32_t what, int64_t value) {
       pl->graphs_refused = false;
       return CLEAN_OK;
     case CLEAN_DEBUG_PLAIN_CYCLES:
-      if (value < 0 || value > (1 << 30) || !pl->mc.resident || !takeover_possible(pl->d))
+      if (value < 0 || value > (1 << 30) || !pl->mc.resident || !takeover_possible(pl->d, pl->p.niter))
         return CLEAN_ERR_INVALID_ARG;
       pl->d.sel.plain_cycles = (float)value;
       return CLEAN_OK;

@@ -217,9 +217,10 @@ __host__ __device__ __forceinline__ bool feedback_on(const PlanDev& d) {
   return (d.K > 0 || d.trigger > 0.f) && d.T > 1;
 }
 // Rounds of several selections, which the plain loop may take over in groups that
-// hold their tile in shared memory (rounds that a flux trigger ends are short: an
-// idle launch each would cost 3 %).
-inline bool takeover_possible(const PlanDev& d) {
+// hold their tile in shared memory.  An idle launch costs 10 us: not for rounds that
+// a flux trigger ends (3 %), nor for runs of a few selections.
+inline bool takeover_possible(const PlanDev& d, int64_t niter) {
+  if (niter / d.T < 256) return false;
   return d.T == 1 ? d.K == 0 || d.K > kSelPending : d.K > kSelPending && !(d.trigger > 0.f);
 }
 // r_map / p_map: 2-D tensor maps of the residual and the PSF with the box

@@ -59,8 +59,9 @@ def test_handed_over_rounds_equal_the_oracle(ny, nx, tiles, K, niter, thr, trigg
 def test_no_hand_over_where_the_plan_has_no_such_launch():
     dirty, psf = _field(64, 64, 5, 1)
     import torch
-    for kw in (dict(tiles=(2, 2), feedback_interval=50), dict(feedback_interval=64)):
-        with cg.Plan(torch.from_numpy(psf).cuda(), 64, 64, niter=10, **kw) as p:
+    for kw in (dict(tiles=(2, 2), feedback_interval=50), dict(feedback_interval=64),
+               dict(niter=255)):
+        with cg.Plan(torch.from_numpy(psf).cuda(), 64, 64, **{"niter": 2000, **kw}) as p:
             with pytest.raises(cg.CleanError) as e:
                 p.debug_set(cg.DEBUG_PLAIN_CYCLES, 1)
             assert e.value.status == 1
