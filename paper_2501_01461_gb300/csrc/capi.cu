@@ -877,6 +877,7 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
     req.push_back({(void**)&pl->fft_twx, sizeof(float2) * (size_t)pl->fft_ax.tw_len});
     req.push_back({(void**)&pl->R0, sizeof(float) * (size_t)npix});
   }
+  const size_t n_needed = req.size();
   if (pl->sel_ok) {
     req.push_back({(void**)&pl->d.sel.u, sel_z.cells});
     req.push_back({(void**)&pl->d.sel.masks, sel_z.cells});
@@ -886,21 +887,37 @@ int clean_plan(clean_plan_t* out, const clean_params* p, const float* d_psf, voi
     if (sel_z.hb) req.push_back({(void**)&pl->sel_hb, sel_z.hb});
     req.push_back({(void**)&pl->sel_lobe, sel_z.lobe});
   }
-  size_t total = 0;
-  for (auto& r : req) total += r.bytes;
+  // where the selection's tables (up to a quarter more than the images) do not fit,
+  // the plan does without: the iteration-by-iteration loops need none
+  auto without_tables = [&] {
+    if (!pl->sel_ok) return false;
+    req.resize(n_needed);
+    pl->sel_ok = false;
+    pl->d.sel = SelDev{};
+    return true;
+  };
   const int64_t lim = g_alloc_limit.load();
-  if (lim >= 0 && (int64_t)total > lim) {
+  auto over_limit = [&] {
+    size_t total = 0;
+    for (auto& r : req) total += r.bytes;
+    return lim >= 0 && (int64_t)total > lim;
+  };
+  if (over_limit() && !(without_tables() && !over_limit())) {
     delete pl;
     return CLEAN_ERR_OOM;
   }
   // one allocation, each array at a multiple of 256 bytes: a server makes a plan
   // per job, and twenty allocations and a page of pinned memory cost it 0.3 ms
   // (0.17 + 0.14) and their release 0.35; one costs 0.08 and 0.05
-  size_t arena = 0;
-  for (auto& r : req) arena += (r.bytes + 255) & ~(size_t)255;
-  if (cudaMalloc(&pl->arena, arena) != cudaSuccess) {
+  auto allocate = [&] {
+    size_t arena = 0;
+    for (auto& r : req) arena += (r.bytes + 255) & ~(size_t)255;
+    if (cudaMalloc(&pl->arena, arena) == cudaSuccess) return true;
     pl->arena = nullptr;
     cudaGetLastError();
+    return false;
+  };
+  if (!allocate() && !(without_tables() && allocate())) {
     clean_destroy(pl);
     return CLEAN_ERR_OOM;
   }
