@@ -221,22 +221,30 @@ def aggregate(dist, ms: float, units: float, device=None):
     return float(t.item()), float(u.item())
 
 
-def minor_bytes_per_run(w) -> int:
+def minor_bytes_per_run(w, by_selection: bool = True) -> int:
     """Algorithmic bytes of all minor loops of one run: a round's selection
     reads the residual once (its cells' bounds) and leaves the subtraction to
-    the feedback; the iterations themselves touch a few KB each."""
+    the feedback; the iterations themselves touch a few KB each.  The
+    iteration-by-iteration loop reads a tile's residual and PSF window and
+    writes its residual in each iteration (12 bytes a pixel)."""
     T = w.tiles[0] * w.tiles[1]
+    if not by_selection:
+        return int(12 * w.n * w.n * w.niter // T)
     per_tile = w.niter // T + (1 if w.niter % T else 0)
     k = w.feedback_interval if w.feedback_interval > 0 else per_tile
     return int(-(-per_tile // k) * 4 * w.n * w.n)
 
 
-def feedback_updates_per_run(w) -> int:
+def feedback_updates_per_run(w, by_selection: bool = True) -> int:
     """Pixel-component updates of all feedbacks of one run (threshold 0, every
     tile spends its budget): each component updates every pixel once, those of
-    its own tile too (the selection leaves a round of up to 64 components
-    pending)."""
-    return int(w.niter * w.n * w.n) if w.feedback_interval > 0 else 0
+    its own tile too where the selection leaves a round of up to 64 components
+    pending, else those of the other tiles."""
+    if w.feedback_interval <= 0:
+        return 0
+    T = w.tiles[0] * w.tiles[1]
+    own = by_selection and w.feedback_interval <= 64
+    return int(w.niter * w.n * w.n * (1 if own else (T - 1) / T))
 
 
 def measured_peaks():
@@ -672,8 +680,10 @@ def main():
     minor_avg = st["minor_ms"] / max(st["minor_launches"], 1)
     fb_avg = st["feedback_ms"] / max(st["feedback_launches"], 1)
     rounds_per_run = st["minor_launches"] / args.steps
-    minor_b = minor_bytes_per_run(w) / rounds_per_run           # per launch
-    fb_upd = feedback_updates_per_run(w) / rounds_per_run       # per launch
+    info = plan.minor_info()
+    sel = info["by_selection"]
+    minor_b = minor_bytes_per_run(w, sel) / rounds_per_run      # per launch
+    fb_upd = feedback_updates_per_run(w, sel) / rounds_per_run  # per launch
     fb_b = 8.0 * w.n * w.n + 4.0 * fb_upd                       # per launch
     minor_gbs = minor_b / (minor_avg / 1e3) / 1e9
     fb_gbs = fb_b / (fb_avg / 1e3) / 1e9
@@ -682,7 +692,13 @@ def main():
     alu_peak = st["sm_count"] * 128 * sm_mhz * 1e6 / 1e12
     rec = ncu_traffic()
     traffic = {k: v["bytes_per_launch"] for k, v in rec.items()}
-    minor_name = "select_kernel"
+    minor_name = ("select_kernel" if sel else "minor_pair_kernel" if st["minor_pairs"] else
+                  "minor_pipe_kernel" if st["minor_pipe"] else "minor_kernel")
+    minor_note = ("the residual once a round over the measured L2 read peak; the launch is "
+                  "bound by the chain of its iterations (us_per_iteration: of one tile, all "
+                  "tiles at once)" if sel else
+                  "12 B per pixel-iteration over the measured L2 read peak; residual rows that "
+                  "stay in shared or tensor memory do not reach L2")
     fb_name = "feedback_tma_kernel" if st["feedback_tma"] else "feedback_kernel"
     l2_src = (f"measured in this run: {l2['form']} ({l2['method']}); MEASURED_PEAKS.json "
               f"holds no L2 figure (its HBM copy peak is {peaks['hbm_gbs']:.0f} GB/s, {peak_src})")
@@ -701,8 +717,7 @@ def main():
         roof = {"kernel": minor_name, "bound": "l2", "achieved": minor_gbs, "peak": l2_gbs,
                 "unit": "GB/s", "frac": minor_gbs / l2_gbs, "traffic": traffic.get(minor_name),
                 "peak_source": l2_src, "bytes_per_launch": minor_b,
-                "note": "the residual once a round; the launch is bound by the chain of its "
-                        "iterations, not by bytes"}
+                "note": minor_note}
     kernels = {
         "minor": {"kernel": minor_name,
                   "ms_per_step": st["minor_ms"] / args.steps,
@@ -712,9 +727,7 @@ def main():
                   "traffic": traffic.get(minor_name),
                   "us_per_iteration": st["minor_ms"] * 1e3 * w.tiles[0] * w.tiles[1]
                   / (w.niter * args.steps),
-                  "note": "the residual once a round over the measured L2 read peak; the "
-                          "launch is bound by the chain of its iterations (us_per_iteration: "
-                          "of one tile, all tiles at once)"},
+                  "note": minor_note},
         "feedback": {"kernel": fb_name,
                      "ms_per_step": st["feedback_ms"] / args.steps,
                      "launches_per_step": st["feedback_launches"] / args.steps,
@@ -846,7 +859,7 @@ def main():
             "data": "synthetic (VLA-like Y array PSF, seeded point-source sky)",
             "config": config_dict(w),
             "px_iter_per_s": value * px_iter,
-            "feedback_px_comp_per_s": world * feedback_updates_per_run(w) * args.steps / (total_ms / 1e3),
+            "feedback_px_comp_per_s": world * feedback_updates_per_run(w, sel) * args.steps / (total_ms / 1e3),
             "roofline": roof, "kernels": kernels, "l2_probe": l2,
             "cpu_baseline": cpu, "cpu_parallel_baseline": cpu_par,
             "e2e": e2e, "untiled_gpu": untiled,
@@ -856,7 +869,8 @@ def main():
             "served": served,
             "gpu_launches": int(gpu_launches),
             "clocks": clocks, "wall_s_timed": wall,
-            "plan": {k: st[k] for k in ("group_ctas", "group_sync", "resident", "sm_count")},
+            "plan": {**info, "sm_count": st["sm_count"],
+                     **({} if sel else {k: st[k] for k in ("group_sync", "resident")})},
         }
         print(json.dumps(line), flush=True)
     plan.close()

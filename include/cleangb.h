@@ -50,8 +50,8 @@
  *     the same code.  No call aborts the process.
  *   - Diagnostics: with the environment variable CLEANGB_REPORT_TIMEOUT set,
  *     the batch and server entry points print to stderr, for each job whose
- *     bounded wait expired, its shape, its unit layout and the tile and
- *     exchange where the wait gave up.
+ *     bounded wait expired, its shape, and the tile and iteration where the
+ *     wait gave up.
  */
 #ifndef CLEANGB_H
 #define CLEANGB_H
@@ -412,11 +412,13 @@ CLEAN_API void clean_destroy(clean_plan_t plan);
 CLEAN_API const char* clean_strerror(int status);
 
 /* Test hooks.  clean_debug_set(plan, what, value):
- *   CLEAN_DEBUG_SPIN_LIMIT_NS  bound (ns) of every grid-barrier wait
- *                              (default 2e9); a wait that exceeds it sets
+ *   CLEAN_DEBUG_SPIN_LIMIT_NS  bound (ns) of every grid-barrier wait and of
+ *                              those of a selection's group (default 2e9); a wait that exceeds it sets
  *                              CLEAN_ERR_TIMEOUT and the kernel returns
- *   CLEAN_DEBUG_FORCE_TIMEOUT  1: the first grid-barrier wait waits for an
- *                              arrival that never comes (it must expire)
+ *   CLEAN_DEBUG_FORCE_TIMEOUT  1: the first grid-barrier wait, or the first
+ *                              of a selection's group, waits for an arrival
+ *                              that never comes (it must expire; a group of one
+ *                              CTA has no wait)
  *   CLEAN_DEBUG_FEEDBACK_PATH  feedback kernel: 0 automatic (TMA when the
  *                              PSF is 16-byte aligned with a row pitch that is
  *                              a multiple of 4 floats), 1 plain loads, 2 TMA

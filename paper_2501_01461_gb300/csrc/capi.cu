@@ -258,7 +258,7 @@ int check_psf(clean_plan_s* pl, cudaStream_t s) {
                           sizeof(float2) * (size_t)pl->d.sel.cell_stride * pl->d.T, s);
     if (e == cudaSuccess)
       e = select_build_psf(pl->d, pl->sel_boxes, pl->sel_h8, pl->sel_hb, pl->sel_lobe, s);
-    pl->kernel_launches += 4;
+    pl->kernel_launches += pl->d.sel.lq > 0 ? 5 : 3;
     if (e != cudaSuccess) return cuda_fail(pl, e);
   }
   rc = read_state(pl, s);
