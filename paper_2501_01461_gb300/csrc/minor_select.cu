@@ -1133,7 +1133,6 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
                                             uint64_t limit_ns, int force_timeout, int t,
                                             int rank) {
   SelShared& s = shared_state();
-  if (*(volatile int32_t*)&d.st->status != 0) return;  // uniform over a launch's start
   const Geo g = make_geo(d, t);
   const uint64_t key = d.peak[parity * d.T + t];
   const int64_t budget = d.budget[t];
@@ -1146,7 +1145,7 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
   const bool hand_all = d.sel.plain_cycles > 0.f && ctl->slow >= kSlowRuns;
   const bool idle = kmax <= 0 || key == 0ull || !(key_abs(key) > d.thr) || !(key_abs(key) > level);
   if (threadIdx.x == 0) {
-    s.abort = 0;
+    s.abort = *(volatile int32_t*)&d.st->status != 0;  // one read for the block
     s.key = 0ull;
     s.slow = ctl->slow;
     if (rank == 0) ctl->hand_key = hand_all && !idle ? key : 0ull;
@@ -1156,6 +1155,7 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
   uint32_t phase = 0;
   bool done = idle;
   __syncthreads();
+  if (s.abort) return;
   while (!idle && !hand_all) {
     if (threadIdx.x == 0) s.t0 = clock64();
     // the pending components, then the cells (unless the round is over)
@@ -1186,7 +1186,7 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
       }
     }
     __syncthreads();
-    if (s.abort) break;
+    if (rank == 0 && s.abort) break;  // (the others' threads 0 may be at its next use)
     if (rank == 0) {
       uint32_t abs0 = (uint32_t)(s.key >> 32), lo0 = (uint32_t)s.key;
       if (phase == 1) {  // the round's first peak is known
