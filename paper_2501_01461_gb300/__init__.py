@@ -172,12 +172,14 @@ def _stream_ptr(stream):
     return ctypes.c_void_p(stream.cuda_stream)
 
 
-def _components(comps, n):
-    """The first n rows of a CUDA int32 array of components as a structured
-    array (the rows are the records, so they are copied once)."""
+def _components(comps, n, stream=None):
+    """The first n rows of a CUDA int32 array of components, written on `stream`,
+    as a structured array (the rows are the records, so they are copied once)."""
+    import torch
     if n == 0:
         return np.empty(0, dtype=COMPONENT_DTYPE)
-    return comps[:n].cpu().numpy().view(COMPONENT_DTYPE).reshape(n)
+    with torch.cuda.stream(stream):  # (None: the current one)
+        return comps[:n].cpu().numpy().view(COMPONENT_DTYPE).reshape(n)
 
 
 def _dptr(t, shape=None, what="tensor"):
@@ -304,7 +306,7 @@ class Plan:
         cnt = ctypes.c_int64(0)
         _check(lib().clean_get(self._h, _dptr(res), _dptr(mod), ctypes.c_void_p(comps.data_ptr()),
                                n, ctypes.byref(cnt), _stream_ptr(stream)), "clean_get")
-        return res, mod, _components(comps, n)
+        return res, mod, _components(comps, n, stream)
 
     def round_offsets(self, stream=None) -> np.ndarray:
         n = ctypes.c_int64(0)
@@ -438,7 +440,7 @@ class Batch:
         _check(lib().clean_batch_get(self._h, int(i), _dptr(res), _dptr(mod),
                                      ctypes.c_void_p(comps.data_ptr()), n.value, ctypes.byref(n),
                                      sp), "clean_batch_get")
-        return res, mod, _components(comps, n.value)
+        return res, mod, _components(comps, n.value, stream)
 
     def graphs(self, enable=None) -> int:
         """Turns CUDA-graph round replay on or off (None: leave as is);

@@ -160,7 +160,7 @@ class Server:
         _check(lib().clean_server_get(self._h, jid, _dptr(res), _dptr(mod),
                                       ctypes.c_void_p(comps.data_ptr()), n.value, ctypes.byref(n),
                                       sp), "clean_server_get")
-        return res, mod, _components(comps, n.value)
+        return res, mod, _components(comps, n.value, self._stream)
 
     def remove(self, jid: int):
         _check(lib().clean_server_remove(self._h, jid), "clean_server_remove")

@@ -37,3 +37,25 @@ def test_no_set_up_work_is_left_on_the_plans_stream(n, tiles, K, mode):
         assert b.query()
         p.run(dirty)
         assert all(torch.equal(g.cpu(), w) for g, w in zip(p.get()[:2], want))
+
+
+def test_results_read_on_another_stream():
+    """The component list comes back on the stream it was copied on, behind the
+    images (16 MB each) that are on their way there."""
+    import torch
+    n = 2048
+    psf = torch.zeros((2 * n, 2 * n), device="cuda")
+    psf[n, n] = 1.0
+    dirty = torch.rand((n, n), device="cuda")
+    s = torch.cuda.Stream()
+    torch.cuda.synchronize()
+    kw = dict(gain=0.5, niter=500)
+    with cg.Plan(psf, n, n, **kw) as p, cg.Batch([dict(psf=psf, ny=n, nx=n, **kw)]) as b:
+        p.run(dirty)
+        want = p.get()[2]
+        assert len(want) == 500
+        for _ in range(5):
+            assert np.array_equal(p.get(stream=s)[2], want)
+        b.run([dirty])
+        torch.cuda.synchronize()
+        assert np.array_equal(b.get(0, stream=s)[2], want)
