@@ -122,9 +122,9 @@ __global__ void validate_psf_kernel(const float* __restrict__ P, int64_t n, int6
 // the terms left out are zeros, so the sums are those of the full convolution
 // bit for bit.  Bound by reading the window while sources are few (2048^2, r 28:
 // 0.098 ms at 0.2 % of the pixels, 2.97 with every sum whole), by the taps of the
-// rows summed whole when they are many (2.2 ms at 40 to 100 %, 0.31 to 0.18 at
-// 256^2; a kernel of lists alone took 14.2 and 3.2 there, one of full sums 2.97
-// and 0.31).
+// rows summed whole when they are many (2.2 ms at 20 to 100 %, 0.18 at 256^2; a
+// kernel of lists alone took 14.2 and 3.2 at 100 %, one of full sums 2.97 and
+// 0.31).
 constexpr int kRList = 2048;         // window pixels looked at in one go, whole rows
 constexpr int kRCounts = kRList / 32;
 // a listed pixel costs about what kRDense taps of a row summed whole cost (between

@@ -48,18 +48,21 @@
 // 20 sources 2.5).  What decides is the run, not its parameters, so rank 0 times
 // its selections: after two running that cost more than the plain loop's
 // iterations (SelDev::plain_cycles) the tile's components are applied, the peak
-// is left in SelCtl::hand_key, and the launch behind this one goes on from there.
-// That field takes 3.05 us now, the sparse one 2.5.
+// is left in SelCtl::hand_key, and the launch behind this one goes on from there
+// (that field 3.05 us, the sparse one 2.5).
 //
-// What bounds it: an iteration is a chain of about 1500 cycles (0.75 us: decode,
-// one L2 round trip of the candidates' PSF gather at one L1 tag a candidate,
-// two warp reductions either side of a barrier), 3400 with superblocks (the
-// gather misses L1 there, and the cells near the peak come after it); the
-// plain loop's were 3.3 us (256^2, cluster of 16) to 12 us (2048^2, and sixteen
-// 1024^2 tiles at once).  On a flat residual the resolved cells' gathers take as
-// long again.  Code size matters: straight-line code beyond the 32 KB that stay
-// near the schedulers ran at a third of the speed, so the rare parts are
-// rolled loops.
+// What bounds it: one CTA a tile selects while its group waits (256^2: 4 % of the
+// group's issue slots, 0.4 % of the L2 rate; sixteen tiles of 1024^2: a round of 50
+// in 0.16 ms and 72 MB).  An iteration is a chain of 1800 cycles with ten clock
+// reads in it: 830 to decode the peak, read the cells' ranges and issue the gather
+// (one L1 tag a candidate), 430 until its values are subtracted, 340 for a warp's
+// reductions, 220 for the barrier and the block's; 3400 with superblocks (the
+// gather misses L1 there, and the cells near the peak come after it).  The plain
+// loop's were 3.3 us (256^2, cluster of 16) to 12 us (2048^2, and sixteen 1024^2
+// tiles at once).  On a flat residual the resolves take as long again (2048^2, 3000
+// iterations: 8.9 of 18 ms, 698 of 16 cells).  Code size matters: straight-line
+// code beyond the 32 KB that stay near the schedulers ran at a third of the speed,
+// so the rare parts are rolled loops.
 #include <algorithm>
 
 #include "cleangb_internal.cuh"
@@ -97,7 +100,7 @@ constexpr uint32_t kLobeMark = 0xffc00000u;
 // a tile goes to the plain loop after this many selections running that cost
 // more than it would, if this many iterations of the round are left (see SelDev)
 constexpr int kSlowRuns = 2, kSlowLeft = 32;
-constexpr float kFollow = 0.75f;
+constexpr float kFollow = 0.75f;  // see slow_above
 constexpr int kUnitRows = 8, kUnitCols = 32;  // pixels a warp takes at a time in a pass
 
 __device__ __forceinline__ uint32_t redux_max(uint32_t v) {
@@ -1120,7 +1123,8 @@ __device__ __forceinline__ bool wait_count(const uint32_t* p, uint32_t want, uin
 
 // The cycles a component above which the plain loop is preferred.  In a batch its
 // launch waits for the last image's selections, so once one has gone over the
-// others follow unless they are a good deal faster.
+// others follow unless they are a good deal faster (32 crowded 200^2 images: 7.8 us
+// an iteration on their own account, now 4.8).
 __device__ __forceinline__ float slow_above(const PlanDev& d) {
   const bool follow = d.sel.handed && *(volatile int32_t*)d.sel.handed > 0;
   return follow ? kFollow * d.sel.plain_cycles : d.sel.plain_cycles;

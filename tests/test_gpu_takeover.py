@@ -85,3 +85,24 @@ def test_crowded_batches_equal_solo_runs():
                 assert np.array_equal(c["y"], o.comps["y"]) and np.array_equal(c["x"], o.comps["x"])
                 assert np.array_equal(r.cpu().numpy().view(np.uint32), o.residual.view(np.uint32))
                 assert np.array_equal(m.cpu().numpy().view(np.uint32), o.model.view(np.uint32))
+
+
+def test_step_of_a_round_that_is_handed_over():
+    """clean_step leaves every component of the round on its own tile, also those
+    that the plain loop found after the hand-over."""
+    import torch
+    dirty, psf = _field(150, 150, 60, 3)
+    with cg.Plan(torch.from_numpy(psf).cuda(), 150, 150, gain=0.1, niter=1600, tiles=(2, 2),
+                 feedback_interval=200) as p:
+        p.debug_set(cg.DEBUG_PLAIN_CYCLES, 1)
+        p.run(torch.from_numpy(dirty).cuda(), max_rounds=0)
+        p.step()
+        r = p.get()[0]
+        o = oracle.clean_f32(dirty, psf, 0.1, 800, 0.0, (2, 2), 0)  # no feedback
+        assert np.array_equal(r.cpu().numpy().view(np.uint32), o.residual.view(np.uint32))
+        assert p.minor_info()["taken_over"] == 4
+        p.feedback()
+        p.run(None)
+        r = p.get()[0]
+        o = oracle.clean_f32(dirty, psf, 0.1, 1600, 0.0, (2, 2), 200)
+        assert np.array_equal(r.cpu().numpy().view(np.uint32), o.residual.view(np.uint32))
