@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <cstddef>
 #include <cstdlib>
 #include <cstring>
 #include <new>
@@ -339,29 +340,29 @@ bool use_select(const clean_plan_s* pl) {
          pl->p.group_sync == CLEAN_SYNC_AUTO;
 }
 
-// A launch of the plain loop behind the selection takes over the tiles on which
+// The plain loop behind the selection takes over the tiles on which
 // a selection turned out slower (minor_select.cu): crowded fields cleaned far
 // into their noise, where most cells come near the peak again and again.
 bool use_takeover(const clean_plan_s* pl) {
   return use_select(pl) && pl->d.sel.plain_cycles > 0.f;
 }
 
-// flush: the residual must hold every component after the launch (a caller
-// may look at it before the feedback).
 MinorCfg takeover_cfg(MinorCfg c) {
   c.takeover = 1;
   return c;
 }
 
-int launch_round_minor(clean_plan_s* pl, cudaStream_t s, bool flush) {
+// flags: kSelFlush where a caller may look at the residual before the feedback;
+// with kSelReport the takeover is left to finish_handed_over.
+int launch_round_minor(clean_plan_s* pl, cudaStream_t s, int flags) {
   const bool pipe = use_pipe(pl);
   const int ev = timed_begin(pl, 0, s);
   cudaError_t e =
-      use_select(pl) ? launch_select(pl->d, pl->sel_G, pl->sel_smem, pl->parity, flush ? 1 : 0,
+      use_select(pl) ? launch_select(pl->d, pl->sel_G, pl->sel_smem, pl->parity, flags,
                                      (uint64_t)pl->mc.spin_limit_ns, pl->mc.force_timeout, s)
                      : launch_minor(pl->d, pipe ? pl->mc_pipe : pl->mc, pl->parity, &pl->r_map,
                                     &pl->p_map_minor, s);
-  if (e == cudaSuccess && use_takeover(pl)) {
+  if (e == cudaSuccess && use_takeover(pl) && !(flags & kSelReport)) {
     e = launch_minor(pl->d, takeover_cfg(pl->mc), pl->parity, nullptr, nullptr, s);
     ++pl->kernel_launches;
   }
@@ -370,6 +371,26 @@ int launch_round_minor(clean_plan_s* pl, cudaStream_t s, bool flush) {
   if (e != cudaSuccess) return cuda_fail(pl, e);
   pl->pending = true;
   return CLEAN_OK;
+}
+
+// The rest of an untiled run whose tile was handed over, once a status read says so
+// (a takeover launched behind every selection cost such runs 10 us): the round is
+// the run's only one, so its first close is taken back and the next one appends the
+// whole list again.
+int finish_handed_over(clean_plan_s* pl, cudaStream_t s) {
+  constexpr size_t from = offsetof(DevState, handed), to = offsetof(DevState, round_comps);
+  cudaError_t e = cudaMemsetAsync(reinterpret_cast<char*>(pl->d.st) + from, 0, to - from, s);
+  if (e != cudaSuccess) return cuda_fail(pl, e);
+  pl->parity ^= 1;
+  --pl->rounds_launched;
+  const int ev = timed_begin(pl, 0, s);
+  e = launch_minor(pl->d, takeover_cfg(pl->mc), pl->parity, nullptr, nullptr, s);
+  timed_end(pl, ev, s);
+  ++pl->kernel_launches;
+  if (e != cudaSuccess) return cuda_fail(pl, e);
+  pl->pending = true;
+  const int rc = launch_round_feedback(pl, s);
+  return rc == CLEAN_OK ? read_state(pl, s) : rc;
 }
 
 // ---- CUDA-graph replay of two rounds --------------------------------------
@@ -559,6 +580,8 @@ int run_rounds(clean_plan_s* pl, int32_t max_rounds, cudaStream_t s) {
     pl->started = false;
     return CLEAN_ERR_NONFINITE;
   }
+  const bool one_round = pl->d.K == 0 && !(pl->d.trigger > 0.f);  // (of one tile, below)
+  const int report = one_round && use_takeover(pl) ? kSelReport : 0;
   int64_t done = 0;
   while (max_rounds < 0 || done < max_rounds) {
     if (!pl->h_st.active) break;
@@ -586,12 +609,13 @@ int run_rounds(clean_plan_s* pl, int32_t max_rounds, cudaStream_t s) {
         }
         if (rc != -1) return rc;
       }
-      if ((rc = launch_round_minor(pl, s, false)) != CLEAN_OK) return rc;
+      if ((rc = launch_round_minor(pl, s, report)) != CLEAN_OK) return rc;
       if ((rc = launch_round_feedback(pl, s)) != CLEAN_OK) return rc;
       ++i;
     }
     done += chunk;
     if ((rc = read_state(pl, s)) != CLEAN_OK) return rc;
+    if (pl->h_st.handed && (rc = finish_handed_over(pl, s)) != CLEAN_OK) return rc;
   }
   return CLEAN_OK;
 }
@@ -1014,7 +1038,7 @@ int clean_step(clean_plan_t pl, void* stream) {
   DeviceGuard g(pl->device);
   cudaStream_t s = as_stream(stream);
   if (pl->pending && (rc = launch_round_feedback(pl, s)) != CLEAN_OK) return rc;
-  return launch_round_minor(pl, s, true);
+  return launch_round_minor(pl, s, kSelFlush);
 }
 
 int clean_feedback(clean_plan_t pl, void* stream) {

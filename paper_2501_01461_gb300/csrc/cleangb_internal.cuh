@@ -72,7 +72,7 @@ struct DevState {
   int32_t status;        // ST_* bits
   int32_t active;        // a tile can run in the next round
   uint32_t fb_done;      // feedback blocks finished (last-block pattern)
-  int32_t pad0;
+  int32_t handed;        // the only round's tile waits for the plain loop (see kSelReport)
   int64_t total;         // components in the list
   int64_t n_rounds;      // rounds recorded (>= 1 component)
   int64_t round_comps;   // components of the last closed round
@@ -85,6 +85,9 @@ struct DevState {
 // Selection minor loop (minor_select.cu): components a selection may leave
 // pending, the control words of a tile's group, and a plan's tables.
 constexpr int kSelPending = 64;
+// launch_select's flags: leave no component pending; report a hand-over in
+// DevState::handed, for a caller that launches the plain loop only then
+enum { kSelFlush = 1, kSelReport = 2 };
 struct SelCtl {
   unsigned long long key[2];  // peak key of a pass, by the pass's parity
   int64_t k;                  // the posted selection: components of the round so far
@@ -218,7 +221,8 @@ __host__ __device__ __forceinline__ bool feedback_on(const PlanDev& d) {
 }
 // Rounds of several selections, which the plain loop may take over in groups that
 // hold their tile in shared memory.  An idle launch costs 10 us: not for rounds that
-// a flux trigger ends (3 %), nor for runs of a few selections.
+// a flux trigger ends (3 %), nor for runs of a few selections.  (A plan whose run is
+// one round of one tile launches the plain loop only when it has to.)
 inline bool takeover_possible(const PlanDev& d, int64_t niter) {
   if (niter / d.T < 256) return false;
   return d.T == 1 ? d.K == 0 || d.K > kSelPending : d.K > kSelPending && !(d.trigger > 0.f);
@@ -245,9 +249,8 @@ bool select_geometry(SelDev* g, int ny, int nx, int ty, int tx, SelSizes* z);
 cudaError_t select_build_psf(const PlanDev& d, float2* boxes, uint32_t* h8, uint32_t* hb,
                              uint32_t* lobe, cudaStream_t s);
 cudaError_t select_prepare();  // kernel attributes
-// One round's minor loops, G CTAs a tile (G > 1: a cooperative launch); flush:
-// leave no component pending.
-cudaError_t launch_select(const PlanDev& d, int G, int smem, int parity, int flush, uint64_t limit_ns,
+// One round's minor loops, G CTAs a tile (G > 1: a cooperative launch).
+cudaError_t launch_select(const PlanDev& d, int G, int smem, int parity, int flags, uint64_t limit_ns,
                           int force_timeout, cudaStream_t s);
 // G CTAs per (image, tile) item (G > 1: a cooperative launch, every CTA on an SM of
 // its own); direct: tiles without superblocks (SelDev::lq 0).

@@ -1130,10 +1130,9 @@ __device__ __forceinline__ float slow_above(const PlanDev& d) {
   return follow ? kFollow * d.sel.plain_cycles : d.sel.plain_cycles;
 }
 
-// CTA `rank` of the G serving tile t for one round.  flush: leave no
-// component pending.
+// CTA `rank` of the G serving tile t for one round.
 template <bool DIRECT>
-__device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity, int flush,
+__device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity, int flags,
                                             uint64_t limit_ns, int force_timeout, int t,
                                             int rank) {
   SelShared& s = shared_state();
@@ -1142,16 +1141,18 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
   const int64_t budget = d.budget[t];
   const int64_t kmax = (d.K > 0 && (int64_t)d.K < budget) ? (int64_t)d.K : budget;
   const float level = d.trigger > 0.f ? *(volatile float*)&d.st->level : 0.f;
+  const int32_t status = *(volatile int32_t*)&d.st->status;
   SelCtl* ctl = d.sel.ctl + t;
   const uint32_t base = ctl->phases;
+  const int slow = ctl->slow;
   // tiles whose rounds the plain loop has taken over (the group reads this
   // before rank 0 can change it: that is behind its wait for their passes)
-  const bool hand_all = d.sel.plain_cycles > 0.f && ctl->slow >= kSlowRuns;
+  const bool hand_all = d.sel.plain_cycles > 0.f && slow >= kSlowRuns;
   const bool idle = kmax <= 0 || key == 0ull || !(key_abs(key) > d.thr) || !(key_abs(key) > level);
   if (threadIdx.x == 0) {
-    s.abort = *(volatile int32_t*)&d.st->status != 0;  // one read for the block
+    s.abort = status != 0;  // one thread's for the block
     s.key = 0ull;
-    s.slow = ctl->slow;
+    s.slow = slow;
     if (rank == 0) ctl->hand_key = hand_all && !idle ? key : 0ull;
   }
   for (int j = threadIdx.x; j < kPending + 16; j += kThreads) s.comp[j] = make_int4(0, 0, 0, 0);
@@ -1163,7 +1164,7 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
   while (!idle && !hand_all) {
     if (threadIdx.x == 0) s.t0 = clock64();
     // the pending components, then the cells (unless the round is over)
-    if (done && (!flush || k == applied)) break;
+    if (done && (!(flags & kSelFlush) || k == applied)) break;
     tile_pass(d, g, rank, G, (int)(k - applied), !done);
     applied = k;
     if (done) break;
@@ -1207,6 +1208,7 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
           ctl->hand_key = make_key(__uint_as_float(abs0 | (lo0 << 31)),
                                    (g.rc.y0 + (int)(p >> 15)) * d.nx + g.rc.x0 + (int)(p & 0x7fffu));
           if (d.sel.handed) atomicAdd(d.sel.handed, 1);
+          if (flags & kSelReport) d.st->handed = 1;
         }
         done = true;
       } else {
@@ -1238,7 +1240,7 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
       if (s.abort) break;
       k = s.k_cmd;
       done = s.done_cmd != 0;
-      if (!done || flush)
+      if (!done || (flags & kSelFlush))
         for (int j = threadIdx.x; j < (int)(k - applied); j += kThreads) {
           int4 c = __ldcg(reinterpret_cast<const int4*>(
               &d.rcomps[(int64_t)t * d.cap_round + applied + j]));
@@ -1264,8 +1266,8 @@ __device__ __forceinline__ void select_body(const PlanDev& d, int G, int parity,
 
 template <bool DIRECT>
 __global__ void __launch_bounds__(kThreads, 1)
-    select_kernel(PlanDev d, int G, int parity, int flush, uint64_t limit_ns, int force_timeout) {
-  select_body<DIRECT>(d, G, parity, flush, limit_ns, force_timeout, (int)blockIdx.x / G,
+    select_kernel(PlanDev d, int G, int parity, int flags, uint64_t limit_ns, int force_timeout) {
+  select_body<DIRECT>(d, G, parity, flags, limit_ns, force_timeout, (int)blockIdx.x / G,
                       (int)blockIdx.x % G);
 }
 
@@ -1447,7 +1449,7 @@ cudaError_t select_prepare() {
   return e;
 }
 
-cudaError_t launch_select(const PlanDev& d, int G, int smem, int parity, int flush,
+cudaError_t launch_select(const PlanDev& d, int G, int smem, int parity, int flags,
                           uint64_t limit_ns, int force_timeout, cudaStream_t s) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)(d.T * G), 1, 1);
@@ -1460,7 +1462,7 @@ cudaError_t launch_select(const PlanDev& d, int G, int smem, int parity, int flu
   cfg.attrs = at;
   cfg.numAttrs = G > 1 ? 1 : 0;  // a group of one waits for nobody
   PlanDev dd = d;
-  void* args[] = {&dd, &G, &parity, &flush, &limit_ns, &force_timeout};
+  void* args[] = {&dd, &G, &parity, &flags, &limit_ns, &force_timeout};
   return cudaLaunchKernelExC(
       &cfg, d.sel.lq == 0 ? (const void*)select_kernel<true> : (const void*)select_kernel<false>,
       args);

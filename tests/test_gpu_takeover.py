@@ -42,6 +42,7 @@ def _run(dirty, psf, niter, cycles, **kw):
     (128, 96, (1, 1), 0, 600, 0.0, 0.0, dict(mode=cg.UNTILED_GRID)),
     (150, 150, (2, 2), 100, 3000, 0.0, 0.0, {}),               # round after round, in graphs
     (150, 150, (1, 1), 200, 900, 0.0, 0.3, {}),
+    (150, 150, (1, 1), 0, 900, 0.0, 0.3, {}),                  # several rounds of one tile
 ], ids=lambda v: str(v) if isinstance(v, (int, float, tuple)) else None)
 def test_handed_over_rounds_equal_the_oracle(ny, nx, tiles, K, niter, thr, trigger, kw):
     dirty, psf = _field(ny, nx, 60, ny + nx)
