@@ -1639,8 +1639,7 @@ const void* batch_fn(int G, int resident) {
   if (G > 1)
     return resident ? (const void*)minor_batch_kernel<CLEAN_SYNC_CLUSTER, true>
                     : (const void*)minor_batch_kernel<CLEAN_SYNC_CLUSTER, false>;
-  return resident ? (const void*)minor_batch_kernel<kSyncNone, true>
-                  : (const void*)minor_batch_kernel<kSyncNone, false>;
+  return (const void*)minor_batch_kernel<kSyncNone, true>;  // (one CTA holds its tile)
 }
 }  // namespace
 
