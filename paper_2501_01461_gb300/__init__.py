@@ -175,11 +175,13 @@ def _stream_ptr(stream):
 def _components(comps, n, stream=None):
     """The first n rows of a CUDA int32 array of components, written on `stream`,
     as a structured array (the rows are the records, so they are copied once)."""
-    import torch
     if n == 0:
         return np.empty(0, dtype=COMPONENT_DTYPE)
-    with torch.cuda.stream(stream):  # (None: the current one)
-        return comps[:n].cpu().numpy().view(COMPONENT_DTYPE).reshape(n)
+    if stream is not None:  # (entering a stream takes the host 10 us)
+        import torch
+        with torch.cuda.stream(stream):
+            return _components(comps, n)
+    return comps[:n].cpu().numpy().view(COMPONENT_DTYPE).reshape(n)
 
 
 def _dptr(t, shape=None, what="tensor"):
